@@ -398,9 +398,10 @@ int stego_embed(const uint8_t *d_cover, uint8_t *d_stego, uint64_t cover_bytes,
                                     slot));
     }
     // PAPER2 out of place: one fused pass when the layout allows it
-    if (!inplace && cover_bytes > 0 && p2_fused_ok(d_cover, d_stego, *geom))
-        return cuda_status(p2_embed_fused(d_cover, d_stego, *geom, d_msg, msg_bytes, stats,
-                                          d_result, sh, s, slot));
+    cudaError_t err = cudaSuccess;
+    if (!inplace && cover_bytes > 0 &&
+        p2_embed_fused(d_cover, d_stego, *geom, d_msg, msg_bytes, stats, d_result, s, slot, &err))
+        return cuda_status(err);
     // otherwise copy the cover (out of place), then write the 4N carrying bytes
     if (!inplace && cover_bytes > 0) {
         cudaError_t e = s1_embed(d_cover, d_stego, cover_bytes, 0, nullptr, 0, false, 0, false,

@@ -52,7 +52,7 @@ struct WsHead {
 
 struct DescInfo {
     uint64_t n_bytes; // stream embed: bytes written; stream extract: 8*len
-    uint64_t t_bytes; // stream embed: carrying bytes
+    uint64_t t_bytes; // stream embed: carrying bytes; paper: R | L_last << 32
     uint64_t len;     // stream embed: stream bytes; extract / paper: message bytes
     uint32_t nbits;   // header value
     uint32_t bits;    // kHeader | kVec | kMsgEven | kFunnel
@@ -61,7 +61,8 @@ struct DescInfo {
     uint32_t channels, plane; // misaligned stream embed: channels = Q (funnel word offset)
     uint32_t mode;     // paper layout: one of the kP2* work kinds
     uint32_t per_tile; // paper layout: units, rows or runs per tile
-    uint32_t pad[2];
+    uint32_t nunits;   // paper layout in units: their number (0: another mode)
+    uint32_t flat;     // their head bytes (16 bits), cover shift and plane position
 };
 static_assert(sizeof(DescInfo) == 64, "DescInfo is 64 bytes");
 
@@ -81,7 +82,11 @@ __device__ __forceinline__ uint64_t whole_rounds(uint64_t per)
 {
     return per >= kP2Threads ? per / kP2Threads * kP2Threads : per;
 }
-constexpr uint32_t kChunk = 4u; // tiles per claim
+// Most tiles per claim, of the stream layout and of the paper's (see
+// claim_size): long runs while there are many tiles, so that a large batch pays
+// few set-ups, and single tiles where there are few, so that a small batch
+// spreads over as many CTAs as there are and all end together.
+constexpr uint32_t kChunk = 2u, kPaperChunk = 4u;
 
 // Workspace: head (64 B), aligned-stream, paper and misaligned-stream tile
 // offsets (n+1 each), per-descriptor info (64 B each, 16-byte aligned).
@@ -131,7 +136,7 @@ __device__ __forceinline__ void clear_info(DescInfo &inf)
     inf.nbits = inf.bits = 0;
     inf.W = inf.H = inf.channels = inf.plane = 0;
     inf.mode = inf.per_tile = 0;
-    inf.pad[0] = inf.pad[1] = 0;
+    inf.nunits = inf.flat = 0;
 }
 
 // Paper-layout geometry of a descriptor: channels > 0, plane < channels and
@@ -145,6 +150,9 @@ __device__ __forceinline__ bool paper_geom_ok(const stego_desc &D)
 
 __device__ __forceinline__ void paper_info(const stego_desc &D, DescInfo &inf, uint64_t N)
 {
+    const uint32_t Q = D.geom.width / 4u;
+    const uint64_t R = Q ? (N + Q - 1) / Q : 0u; // as in p2::make_view
+    inf.t_bytes = R | (R ? (N - (R - 1) * Q) << 32 : 0u);
     inf.len = N;
     inf.W = D.geom.width;
     inf.H = D.geom.height;
@@ -207,26 +215,21 @@ __global__ void prep_embed(const stego_desc *descs, uint32_t n, stego_result *re
             const uint64_t rows_per_tile = rows_for(D, tile_bytes);
             const p2::View v = p2::make_view(nullptr, nullptr, D.geom.width, D.geom.height, ch,
                                              D.geom.plane, nullptr, nullptr, D.msg_bytes);
-            if (!inplace && d_aligned16(D.cover) && d_aligned16(D.stego) &&
-                (ch == 3 || ch == 1) && D.geom.width % 16u == 0 &&
-                (uint64_t)D.geom.width / 16u * D.geom.height < (1ull << 31)) {
-                // one-pass units: grayscale, or RGB with any plane
-                const uint64_t units = (uint64_t)(D.geom.width / 16u) * D.geom.height;
+            p2::Flat f;
+            const bool flat = p2::make_flat(D.cover, D.stego, D.cover_bytes, ch, D.geom.plane, true, f);
+            if (flat && (!inplace || (d_aligned16(D.cover) && D.geom.width % 16u == 0))) {
+                // one-pass units, for 1, 3 or 4 channels, any row length and
+                // any addresses; in place (rows of whole vectors, 16-byte
+                // aligned) the units with carrying pixels, written back whole
+                const uint64_t units = inplace ? p2::carrying_units(v, f) : f.nunits;
                 const uint64_t per =
                     whole_rounds(tile_bytes / (16u * ch) ? tile_bytes / (16u * ch) : 1u);
-                inf.mode = kP2Units;
+                inf.mode = inplace ? kP2UnitsInPlace : kP2Units;
                 inf.per_tile = (uint32_t)per;
-                tiles = (units + per - 1) / per;
-            } else if (inplace && d_aligned16(D.cover) && (ch == 3 || ch == 1) &&
-                       D.geom.width % 16u == 0 &&
-                       (uint64_t)D.geom.width / 16u * D.geom.height < (1ull << 31)) {
-                // in place: the units of the carrying rows, written back whole
-                const uint64_t units = (uint64_t)(D.geom.width / 16u) * v.R;
-                const uint64_t per =
-                    whole_rounds(tile_bytes / (16u * ch) ? tile_bytes / (16u * ch) : 1u);
-                inf.mode = kP2UnitsInPlace;
-                inf.per_tile = (uint32_t)per;
-                tiles = (units + per - 1) / per;
+                inf.n_bytes = units;
+                inf.nunits = f.nunits;
+                inf.flat = f.h | (f.d << 16) | (f.ph << 24);
+                tiles = units ? (units + per - 1) / per : 1u; // (at least the edge bytes)
             } else if (!inplace) {
                 inf.mode = kP2RowsCopy;
                 inf.per_tile = (uint32_t)rows_per_tile;
@@ -347,10 +350,10 @@ __global__ void prep_extract(const stego_desc *descs, uint32_t n, stego_result *
         unsigned long long tiles = 0;
         if (layout == STEGO_LAYOUT_PAPER2 && st == STEGO_OK) {
             paper_info(D, inf, len);
-            const p2::View v = p2::make_view(nullptr, nullptr, D.geom.width, D.geom.height,
-                                             D.geom.channels, D.geom.plane, nullptr, nullptr, len);
+            const p2::View v = p2::make_view(D.cover, nullptr, D.geom.width, D.geom.height,
+                                             D.geom.channels, D.geom.plane, nullptr, D.msg, len);
             if (p2::unit_channels(D.geom.channels)) {
-                const uint64_t runs = (uint64_t)((v.Q + 15) / 16) * v.R;
+                const uint64_t runs = p2::run_count(v);
                 const uint64_t per = whole_rounds(tile_bytes / (64u * D.geom.channels)
                                                       ? tile_bytes / (64u * D.geom.channels)
                                                       : 1u);
@@ -499,110 +502,172 @@ __device__ __forceinline__ void flush_stats(unsigned long long &changed, unsigne
     sse = 0;
 }
 
-// The claim loop shared by both directions: calls body(d, local_tile) for
-// every tile this CTA claims, in order.
-template <typename Body>
+// The claim loop shared by both directions: calls body(d, first, count) for
+// the tiles of the chunks this CTA claims, in order.  MERGE: once for every run
+// of `count` consecutive tiles of one descriptor, one set-up for all of them (a
+// call per tile cost the paper layout's kernels as many instructions as a
+// round of their threads); else tile by tile, count = 1 (the stream kernels'
+// set-up is a few loads, and merged ranges cost persist_embed<4, true> two
+// registers and with them the third CTA per SM).
+// Tiles of a claim: a quarter of the CTA's share of `left` tiles, at most MAX.
+template <uint32_t MAX>
+__device__ __forceinline__ uint32_t claim_size(unsigned long long left)
+{
+    const uint32_t n = (left >> 32) ? MAX : (uint32_t)left / (4u * gridDim.x);
+    return n < 1u ? 1u : n < MAX ? n : MAX;
+}
+
+template <bool MERGE, typename Body>
 __device__ __forceinline__ void claim_loop(const unsigned long long *start,
                                            unsigned long long total,
                                            unsigned long long *counter, uint32_t n, Body &&body)
 {
+    constexpr uint32_t MAX = MERGE ? kPaperChunk : kChunk;
     __shared__ unsigned long long s_claim;
-    if (threadIdx.x == 0)
-        s_claim = atomicAdd(counter, (unsigned long long)kChunk);
+    __shared__ uint32_t s_count;
+    if (threadIdx.x == 0) {
+        const uint32_t cnt = claim_size<MAX>(total);
+        s_count = cnt;
+        s_claim = atomicAdd(counter, (unsigned long long)cnt);
+    }
     __syncthreads();
     for (;;) {
-        const unsigned long long c0 = s_claim;
+        const unsigned long long c0 = s_claim, ce = c0 + s_count;
         __syncthreads(); // every thread has read the claim
         if (c0 >= total)
             break;
-        if (threadIdx.x == 0) // next claim in flight while this chunk runs
-            s_claim = atomicAdd(counter, (unsigned long long)kChunk);
-        const unsigned long long c1 = c0 + kChunk < total ? c0 + kChunk : total;
+        const unsigned long long c1 = ce < total ? ce : total;
+        if (threadIdx.x == 0) { // next claim in flight while this chunk runs
+            const uint32_t cnt = claim_size<MAX>(total - c1);
+            s_count = cnt;
+            s_claim = atomicAdd(counter, (unsigned long long)cnt);
+        }
         uint32_t d = owner_of(start, n, c0);
-        for (unsigned long long t = c0; t < c1; ++t) {
-            while (start[d + 1] <= t)
-                ++d;
-            body(d, t - start[d]);
+        if constexpr (MERGE) {
+            unsigned long long t = c0;
+            while (t < c1) {
+                while (start[d + 1] <= t)
+                    ++d;
+                const uint32_t cnt = (uint32_t)((start[d + 1] < c1 ? start[d + 1] : c1) - t);
+                t += cnt;
+                body(d, t - cnt - start[d], cnt);
+            }
+        } else {
+            for (unsigned long long t = c0; t < c1; ++t) {
+                while (start[d + 1] <= t)
+                    ++d;
+                body(d, t - start[d], 1u);
+            }
         }
         __syncthreads(); // the next claim is visible
     }
 }
 
-struct TileStats {
-    unsigned long long changed, sse;
+// What the CTA's threads need to know of a paper-layout cover, in shared memory:
+// read where it is used, it costs the routines below no registers (passed by
+// value it lay on each thread's stack, and a quarter of the instructions
+// were its loads and stores).
+struct PaperJob {
+    p2::View v;
+    p2::Flat f;
 };
 
-// The units of one tile of an RGB cover carrying in plane PLANE.
-template <int PLANE, bool STATS>
-__device__ __noinline__ TileStats rgb_units_tile(const p2::View v, uint32_t k0, uint32_t k1)
+__device__ __forceinline__ const PaperJob &paper_job(const stego_desc &D, const DescInfo &inf,
+                                                     bool embed)
 {
-    TileStats t{0ull, 0ull};
-    p2::units_embed<3, PLANE, STATS, 1>(v, k0, k1, blockDim.x, t.changed, t.sse);
-    return t;
+    __shared__ PaperJob job;
+    __syncthreads(); // every thread is done with the previous cover
+    if (threadIdx.x == 0) {
+        p2::View &v = job.v;
+        v.src = D.cover;
+        v.dst = embed ? D.stego : nullptr;
+        v.msg_in = embed ? D.msg : nullptr;
+        v.msg_out = embed ? nullptr : D.msg;
+        v.N = inf.len;
+        v.W = inf.W;
+        v.H = inf.H;
+        v.channels = inf.channels;
+        v.plane = inf.plane;
+        v.Q = inf.W / 4u;
+        v.R = (uint32_t)inf.t_bytes;
+        v.L_last = (uint32_t)(inf.t_bytes >> 32);
+        v.kmul = 4u;
+        job.f.h = inf.flat & 0xFFFFu;
+        job.f.d = (inf.flat >> 16) & 0xFFu;
+        job.f.ph = inf.flat >> 24;
+        job.f.x0 = inf.channels == 1 ? job.f.h
+                                     : (job.f.h + job.f.ph - inf.plane) / inf.channels;
+        job.f.nunits = inf.nunits;
+        job.f.sel = p2::make_sel(inf.channels, job.f.ph);
+    }
+    __syncthreads();
+    return job;
 }
 
-// One tile of a paper-layout cover (the CTA's threads together).
+// Tiles lt .. lt + cnt - 1 of a paper-layout cover (the CTA's threads together).
 template <bool STATS>
 __device__ __forceinline__ void paper_embed_tile(const stego_desc &D, const DescInfo &inf,
-                                                 unsigned long long lt,
+                                                 unsigned long long lt, uint32_t cnt,
                                                  unsigned long long &changed,
                                                  unsigned long long &sse)
 {
-    const p2::View v = p2::make_view(D.cover, D.stego, inf.W, inf.H, inf.channels, inf.plane,
-                                     D.msg, nullptr, inf.len);
-    const uint64_t b0 = lt * inf.per_tile, b1 = b0 + inf.per_tile;
+    const PaperJob &job = paper_job(D, inf, true);
+    const uint64_t b0 = lt * inf.per_tile, b1 = b0 + (uint64_t)cnt * inf.per_tile;
     if (inf.mode == kP2Units || inf.mode == kP2UnitsInPlace) {
         // in place the same code runs over the carrying rows' units only:
         // each unit is read and written back by one thread, so src == dst is
         // safe, and the last row's units past its carrying columns are
         // rewritten unchanged (one instantiation keeps the registers down)
-        const bool ip = inf.mode == kP2UnitsInPlace;
-        const uint64_t units = (uint64_t)(inf.W / 16u) * (ip ? v.R : inf.H);
         const uint32_t k0 = (uint32_t)b0 + threadIdx.x;
-        const uint32_t k1 = (uint32_t)(b1 < units ? b1 : units);
+        const uint32_t k1 = (uint32_t)(b1 < inf.n_bytes ? b1 : inf.n_bytes);
         // one unit per thread, loaded by the thread itself: under the
         // 80-register cap a form staged through shared memory spilled more
         // and ran slower (600 video frames: 1.53 against 1.26 ms), and so did
         // the cp.async pipeline of the single-cover kernel (1.34-1.83 ms)
-        if (inf.channels == 1) {
-            p2::units_embed<1, 0, STATS, 1>(v, k0, k1, blockDim.x, changed, sse);
-        } else if (inf.plane == 0) {
-            p2::units_embed<3, 0, STATS, 1>(v, k0, k1, blockDim.x, changed, sse);
-        } else {
-            // planes 1 and 2 of RGB in calls of their own, so that their
-            // registers do not crowd the plane-0 path (once per tile)
-            const TileStats t = inf.plane == 1 ? rgb_units_tile<1, STATS>(v, k0, k1)
-                                               : rgb_units_tile<2, STATS>(v, k0, k1);
-            changed += t.changed;
-            sse += t.sse;
+        switch (inf.channels) {
+        case 1: p2::units_embed<1, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
+        case 3: p2::units_embed<3, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
+        default: p2::units_embed<4, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
         }
+        if (b0 == 0 || b1 >= inf.n_bytes)
+            p2::edge_bytes<STATS>(job.v, job.f, b0 == 0, b1 >= inf.n_bytes, changed, sse);
         return;
     }
     const uint32_t r0 = (uint32_t)b0;
     const uint32_t r1 = (uint32_t)(b1 < inf.H ? b1 : inf.H);
     if (inf.mode == kP2RowsCopy) {
-        p2::rows_copy(v, r0, r1);
+        p2::rows_copy(job.v, r0, r1);
         __syncthreads(); // the copy lands before the scatter overwrites plane bytes
     }
-    p2::rows_embed<STATS>(v, r0, r1, 1, changed, sse);
+    p2::rows_embed<STATS>(job.v, r0, r1, 1, changed, sse);
 }
 
+// a run's quarters whose vectors are in flight together, in aligned layouts
+// and others
+constexpr int kBatchAligned = 2, kBatchQuarters = 1;
+
 __device__ __forceinline__ void paper_extract_tile(const stego_desc &D, const DescInfo &inf,
-                                                   unsigned long long lt)
+                                                   unsigned long long lt, uint32_t cnt)
 {
-    const p2::View v = p2::make_view(D.cover, nullptr, inf.W, inf.H, inf.channels, inf.plane,
-                                     nullptr, D.msg, inf.len);
-    const uint64_t b0 = lt * inf.per_tile, b1 = b0 + inf.per_tile;
+    const PaperJob &job = paper_job(D, inf, false);
+    const uint64_t b0 = lt * inf.per_tile, b1 = b0 + (uint64_t)cnt * inf.per_tile;
     if (inf.mode == kP2Runs) {
-        const uint64_t runs = (uint64_t)((v.Q + 15) / 16) * v.R;
-        p2::runs_extract_any(v, b0 + threadIdx.x, b1 < runs ? b1 : runs, blockDim.x);
+        const uint64_t runs = p2::run_count(job.v);
+        const uint64_t k0 = b0 + threadIdx.x, k1 = b1 < runs ? b1 : runs;
+        switch (inf.channels) {
+        case 1: p2::runs_extract<1, 4, 1>(job.v, k0, k1, blockDim.x); break;
+        case 3: p2::runs_extract<3, kBatchAligned, kBatchQuarters>(job.v, k0, k1, blockDim.x); break;
+        default: p2::runs_extract<4, kBatchAligned, kBatchQuarters>(job.v, k0, k1, blockDim.x); break;
+        }
     } else {
-        p2::rows_extract(v, (uint32_t)b0, (uint32_t)(b1 < v.R ? b1 : v.R), 1);
+        p2::rows_extract(job.v, (uint32_t)b0, (uint32_t)(b1 < job.v.R ? b1 : job.v.R), 1);
     }
 }
 
-template <int V, bool STATS>
-__global__ void __launch_bounds__(512) persist_embed(const stego_desc *descs, uint32_t n,
+// Four vectors per thread in CTAs of at most 256 threads (the default shape)
+// keep 80 registers, three CTAs per SM: 82 cost 13% of the uneven batch.
+template <int V, bool STATS, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 1) persist_embed(const stego_desc *descs, uint32_t n,
                                                      stego_result *results, WsView ws,
                                                      uint32_t tile_bytes)
 {
@@ -610,8 +675,8 @@ __global__ void __launch_bounds__(512) persist_embed(const stego_desc *descs, ui
     allow_dependents();
     unsigned long long changed = 0, sse = 0;
     uint32_t stat_d = 0xFFFFFFFFu;
-    claim_loop(ws.start, ws.head->total, &ws.head->counter, n,
-               [&](uint32_t d, unsigned long long lt) {
+    claim_loop<false>(ws.start, ws.head->total, &ws.head->counter, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
             stat_d = d;
@@ -629,8 +694,8 @@ __global__ void __launch_bounds__(512) persist_embed(const stego_desc *descs, ui
         a.nbits = inf.nbits;
         a.msg_even = (inf.bits & kMsgEven) ? 1u : 0u;
         a.pad = 0;
-        const uint64_t b0 = lt * tile_bytes;
-        const uint64_t b1 = b0 + tile_bytes < inf.n_bytes ? b0 + tile_bytes : inf.n_bytes;
+        const uint64_t b0 = lt * tile_bytes, be = b0 + (uint64_t)cnt * tile_bytes;
+        const uint64_t b1 = be < inf.n_bytes ? be : inf.n_bytes;
         if (inf.bits & kVec) {
             s1::embed_vec_range<V, STATS>(a, (b0 >> 4) + threadIdx.x, b1 >> 4,
                                           (uint64_t)blockDim.x * V, changed, sse);
@@ -651,8 +716,8 @@ __global__ void __launch_bounds__(512) persist_extract(const stego_desc *descs, 
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
-    claim_loop(ws.start, ws.head->total, &ws.head->counter, n,
-               [&](uint32_t d, unsigned long long lt) {
+    claim_loop<false>(ws.start, ws.head->total, &ws.head->counter, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         const stego_desc &D = descs[d];
         const DescInfo inf = ws.info[d];
         s1::ExtractView x;
@@ -662,8 +727,8 @@ __global__ void __launch_bounds__(512) persist_extract(const stego_desc *descs, 
         x.base = (inf.bits & kHeader) ? 32u : 0u;
         x.msg_even = (inf.bits & kMsgEven) ? 1u : 0u;
         x.pad = 0;
-        const uint64_t b0 = lt * tile_bytes;
-        const uint64_t b1 = b0 + tile_bytes < inf.n_bytes ? b0 + tile_bytes : inf.n_bytes;
+        const uint64_t b0 = lt * tile_bytes, be = b0 + (uint64_t)cnt * tile_bytes;
+        const uint64_t b1 = be < inf.n_bytes ? be : inf.n_bytes;
         if (inf.bits & kVec) {
             s1::extract_vec_range<V>(x, (b0 >> 4) + threadIdx.x, b1 >> 4, (uint64_t)blockDim.x * V);
             if (b1 == inf.n_bytes && (x.len & 1u) && threadIdx.x == 0)
@@ -696,10 +761,10 @@ __device__ __forceinline__ void mis_funnel(const s1::EmbedView &a, uint32_t h, u
                                                  blockDim.x >> 5, changed, sse);
 }
 
-// One tile of a misaligned stream cover (the CTA's threads together).
+// Tiles lt .. lt + cnt - 1 of a misaligned stream cover (the CTA's threads together).
 template <bool STATS>
 __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescInfo &inf,
-                                               unsigned long long lt,
+                                               unsigned long long lt, uint32_t cnt,
                                                unsigned long long &changed,
                                                unsigned long long &sse)
 {
@@ -716,8 +781,8 @@ __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescIn
         a.pad = 0;
         const uint32_t h = inf.W;
         const uint64_t nvb = (inf.n_bytes - h) >> 4;
-        const uint64_t j0 = lt * inf.per_tile;
-        const uint64_t j1 = j0 + inf.per_tile < nvb ? j0 + inf.per_tile : nvb;
+        const uint64_t j0 = lt * inf.per_tile, je = j0 + (uint64_t)cnt * inf.per_tile;
+        const uint64_t j1 = je < nvb ? je : nvb;
         if (inf.bits & kFunnel) {
             switch (inf.channels) {
             case 0: mis_funnel<0, STATS>(a, h, inf.H, j0, j1, changed, sse); break;
@@ -744,7 +809,7 @@ __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescIn
 }
 
 __device__ __forceinline__ void mis_extract_tile(const stego_desc &D, const DescInfo &inf,
-                                                 unsigned long long lt)
+                                                 unsigned long long lt, uint32_t cnt)
 {
         s1::ExtractView x;
         x.st = D.cover;
@@ -754,8 +819,8 @@ __device__ __forceinline__ void mis_extract_tile(const stego_desc &D, const Desc
         x.msg_even = (inf.bits & kMsgEven) ? 1u : 0u;
         x.pad = 0;
         const uint64_t np = inf.len >> 1;
-        const uint64_t p0 = lt * inf.per_tile;
-        const uint64_t p1 = p0 + inf.per_tile < np ? p0 + inf.per_tile : np;
+        const uint64_t p0 = lt * inf.per_tile, pe = p0 + (uint64_t)cnt * inf.per_tile;
+        const uint64_t p1 = pe < np ? pe : np;
         s1::extract_shift_lsb<kMisXV>(x, D.cover_bytes, p0, p1, threadIdx.x >> 5,
                                       blockDim.x >> 5);
         if (p1 == np && (x.len & 1u) && threadIdx.x == 0)
@@ -785,13 +850,13 @@ __global__ void __launch_bounds__(kMisEmbedThreads, kMisEmbedMinCtas)
     allow_dependents();
     unsigned long long changed = 0, sse = 0;
     uint32_t stat_d = 0xFFFFFFFFu;
-    claim_loop(ws.start_m, ws.head->total_m, &ws.head->counter_m, n,
-               [&](uint32_t d, unsigned long long lt) {
+    claim_loop<false>(ws.start_m, ws.head->total_m, &ws.head->counter_m, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
             stat_d = d;
         }
-        mis_embed_tile<STATS>(descs[d], ws.info[d], lt, changed, sse);
+        mis_embed_tile<STATS>(descs[d], ws.info[d], lt, cnt, changed, sse);
     });
     if (STATS)
         flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
@@ -802,57 +867,65 @@ __global__ void __launch_bounds__(kMisExtractThreads)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
-    claim_loop(ws.start_m, ws.head->total_m, &ws.head->counter_m, n,
-               [&](uint32_t d, unsigned long long lt) {
-        mis_extract_tile(descs[d], ws.info[d], lt);
+    claim_loop<false>(ws.start_m, ws.head->total_m, &ws.head->counter_m, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
+        mis_extract_tile(descs[d], ws.info[d], lt, cnt);
     });
 }
 
 // The paper layout's own persistent kernels (a separate register budget from
 // the stream kernels): tiles of units, rows or runs, claimed like above.
-// Capped at 80 registers for three CTAs per SM: on 600 video frames the
-// embed with statistics went from 1.47 to 1.32 ms and the extract from 0.54
-// to 0.48 ms, although the statistics variant spills (120 bytes).
+// Capped at 64 registers for four CTAs per SM (1024 covers of sides 64 to 4096,
+// half RGB: embed 960 us against 1023 with three CTAs at 80 registers, 1107
+// with two, although it spills; extract 381 against 410).  One unit or run at a
+// time: with four CTAs the warps hide the latency, and two in flight were
+// slower.  With rows that are not whole vectors copied and then scattered byte
+// by byte the same batch took 2824 us (embed) and 505 us (extract), now 900
+// and 395; large RGB covers run at 0.75 of the copy rate, gray ones, with
+// three times the units per byte, at 0.53.
 template <bool STATS>
-__global__ void __launch_bounds__(kP2Threads, 3) persist_p2_embed(const stego_desc *descs, uint32_t n,
+__global__ void __launch_bounds__(kP2Threads, 4) persist_p2_embed(const stego_desc *descs, uint32_t n,
                                                         stego_result *results, WsView ws)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
     unsigned long long changed = 0, sse = 0;
     uint32_t stat_d = 0xFFFFFFFFu;
-    claim_loop(ws.start_p, ws.head->total_p, &ws.head->counter_p, n,
-               [&](uint32_t d, unsigned long long lt) {
+    claim_loop<true>(ws.start_p, ws.head->total_p, &ws.head->counter_p, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
             stat_d = d;
         }
-        paper_embed_tile<STATS>(descs[d], ws.info[d], lt, changed, sse);
+        paper_embed_tile<STATS>(descs[d], ws.info[d], lt, cnt, changed, sse);
     });
     if (STATS)
         flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
 }
 
-__global__ void __launch_bounds__(kP2Threads, 3) persist_p2_extract(const stego_desc *descs, uint32_t n,
+__global__ void __launch_bounds__(kP2Threads, 4) persist_p2_extract(const stego_desc *descs, uint32_t n,
                                                           WsView ws)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
-    claim_loop(ws.start_p, ws.head->total_p, &ws.head->counter_p, n,
-               [&](uint32_t d, unsigned long long lt) {
-        paper_extract_tile(descs[d], ws.info[d], lt);
+    claim_loop<true>(ws.start_p, ws.head->total_p, &ws.head->counter_p, n,
+               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
+        paper_extract_tile(descs[d], ws.info[d], lt, cnt);
     });
 }
 
 template <bool EMBED>
-const void *persist_kernel(int vec, bool stats)
+const void *persist_kernel(int vec, int threads, bool stats)
 {
     if (EMBED) {
         switch (vec) {
-        case 1: return stats ? (const void *)persist_embed<1, true> : (const void *)persist_embed<1, false>;
-        case 2: return stats ? (const void *)persist_embed<2, true> : (const void *)persist_embed<2, false>;
-        case 8: return stats ? (const void *)persist_embed<8, true> : (const void *)persist_embed<8, false>;
-        default: return stats ? (const void *)persist_embed<4, true> : (const void *)persist_embed<4, false>;
+        case 1: return stats ? (const void *)persist_embed<1, true, false> : (const void *)persist_embed<1, false, false>;
+        case 2: return stats ? (const void *)persist_embed<2, true, false> : (const void *)persist_embed<2, false, false>;
+        case 8: return stats ? (const void *)persist_embed<8, true, false> : (const void *)persist_embed<8, false, false>;
+        default:
+            if (threads <= 256)
+                return stats ? (const void *)persist_embed<4, true, true> : (const void *)persist_embed<4, false, true>;
+            return stats ? (const void *)persist_embed<4, true, false> : (const void *)persist_embed<4, false, false>;
         }
     }
     switch (vec) {
@@ -910,7 +983,7 @@ int batched(const stego_desc *d_descs, uint32_t n, stego_result *d_results, uint
         return STEGO_E_CUDA;
 
     const bool stats = (flags & STEGO_FUSE_STATS) != 0;
-    const void *k = persist_kernel<EMBED>(sh.vec, stats);
+    const void *k = persist_kernel<EMBED>(sh.vec, sh.threads, stats);
     // the tile count lives on the device: launch the full persistent grid
     const int grid = persistent_grid(k, sh.threads, 0, sh.ctas_per_sm, ~0ull >> 1, 1);
     if (EMBED) {

@@ -136,13 +136,14 @@ cudaError_t p2_embed(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
 cudaError_t p2_extract(const uint8_t *st, const stego_geom &g, uint8_t *msg, uint64_t N,
                        stego_result *res, const Shape &sh, cudaStream_t s);
 
-// PAPER2 out of place in one pass (copy and embed fused); usable when
-// p2_fused_ok: distinct 16-byte aligned buffers, 1, 3 or 4 channels and
-// 16-byte aligned rows.  N may be 0 (a copy).
-bool p2_fused_ok(const uint8_t *cover, const uint8_t *stego, const stego_geom &g);
-cudaError_t p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
-                           const uint8_t *msg, uint64_t N, bool stats, stego_result *res,
-                           const Shape &sh, cudaStream_t s, StatSlot *slot = nullptr);
+// PAPER2 out of place in one pass (copy and embed fused), for 1, 3 or 4
+// channels: any row length and any addresses.  N may be 0 (a copy).  Returns
+// false with nothing launched when the layout is not one of these (another
+// channel count, an image of less than a few vectors); else *err is the
+// launch's error.
+bool p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
+                    const uint8_t *msg, uint64_t N, bool stats, stego_result *res,
+                    cudaStream_t s, StatSlot *slot, cudaError_t *err);
 
 // STREAM1 with k = 1..4 bits per carrying byte, over all bytes or one plane
 // (k >= 2 or plane_only; k = 1 over all bytes is s1_embed).
@@ -276,6 +277,55 @@ __device__ __forceinline__ void word_stats(uint32_t x, uint32_t y, unsigned long
     changed += __popc(d & 0x01010101u);
     const uint32_t a = __vabsdiffu4(x, y);
     sse += __dp4a(a, a, 0u);
+}
+
+// Changed bytes and squared error of a unit's 16 carrying bytes (c before,
+// o after, d = o ^ c, differences in the low K bits only), summed in 32 bits
+// per unit.  A byte changed when any of its low K bits did (the packing and
+// the per-field test are below).  With K = 1 every change is +-1, so the
+// squared error equals the count.
+template <int K>
+__device__ __forceinline__ void unit_stats(const uint32_t (&o)[4], const uint32_t (&c)[4],
+                                           const uint32_t (&d)[4], uint32_t kmul,
+                                           unsigned long long &changed,
+                                           unsigned long long &sse)
+{
+    constexpr uint32_t BM = ((1u << K) - 1u) * 0x01010101u;
+    uint32_t n, s = 0;
+    static_assert(K >= 1 && K <= 4, "one to four bits per byte");
+    if constexpr (K <= 2) {
+        // the four words' K-bit changes in disjoint bit ranges of each byte
+        // (word i at bits K*i), joined by multiply-adds, then one fold
+        // Horner in kmul = 1 << K: multiply-adds (FMA pipe), not shifts on
+        // the busy ALU pipe; kmul comes from the launch arguments so the
+        // compiler keeps the multiplies
+        const uint32_t acc0 = ((d[3] * kmul + d[2]) * kmul + d[1]) * kmul + d[0];
+        uint32_t acc = acc0;
+        if (K == 2)
+            acc = (acc | (acc >> 1)) & 0x55555555u;
+        n = __popc(acc);
+    } else {
+        // k = 3, 4: two words per byte (word 2j+1 at bit K), then a field is
+        // nonzero when its top bit is set or its low K-1 bits plus all ones
+        // carry into the top bit (no carry leaves a field)
+        constexpr uint32_t LOW = K == 4 ? 0x77777777u : 0x1B1B1B1Bu;
+        constexpr uint32_t TOP = K == 4 ? 0x88888888u : 0x24242424u;
+        const uint32_t a01 = d[1] * kmul + d[0], a23 = d[3] * kmul + d[2];
+        n = __popc((a01 | ((a01 & LOW) + LOW)) & TOP) + __popc((a23 | ((a23 & LOW) + LOW)) & TOP);
+    }
+    if (K > 1) {
+        uint32_t ab = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { // sum of (a - b)^2 = a.a + b.b - 2 a.b over the fields
+            const uint32_t fa = o[i] & BM, fb = c[i] & BM;
+            s = __dp4a(fa, fa, s);
+            s = __dp4a(fb, fb, s);
+            ab = __dp4a(fa, fb, ab);
+        }
+        s -= 2u * ab;
+    }
+    changed += n;
+    sse += K > 1 ? s : n;
 }
 
 // Warp staging of pixel units (16 pixels of CH channels = CH 16-byte

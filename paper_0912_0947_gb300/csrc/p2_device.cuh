@@ -10,12 +10,13 @@
 // pairs back (Section VII step 6).
 //
 // Work units:
-//   unit  16 consecutive pixels of a row = CH 16-byte vectors (rows of whole
-//         vectors, CH in {1,3,4}); pixel t keeps its plane byte at unit byte
-//         t*CH + PLANE, a compile-time position.  One-pass out-of-place
-//         embedding (2C + N bytes).
-//   run   16 consecutive message bytes of a row: extraction reads the four
-//         units at columns i*L + j0 and ORs their pairs.
+//   unit  16 * CH consecutive stego bytes from a 16-byte boundary on (CH in
+//         {1,3,4} channels): CH whole vectors, which hold the plane bytes of
+//         16 consecutive pixels at the same unit bytes everywhere, whatever the row length and the buffers' addresses (see
+//         Flat).  One-pass out-of-place embedding (2C + N bytes).
+//   run   the message bytes of one row in one 16-byte block of the output:
+//         extraction reads the 16 pixels at columns i*L + j of each quarter
+//         i as the aligned vectors around them and ORs their pairs.
 //   row   thread j of a row handles B[r*Q + j] and its four plane bytes (any
 //         channel count; in place; after a copy out of place).
 #pragma once
@@ -36,7 +37,7 @@ struct View {
     uint32_t Q;      // bytes per full row, floor(W/4)
     uint32_t R;      // rows that carry data
     uint32_t L_last; // bytes in row R-1
-    uint32_t pad;
+    uint32_t kmul;   // 4, a multiplier the compiler cannot see (see unit_stats)
 };
 
 __host__ __device__ inline View make_view(const uint8_t *src, uint8_t *dst, uint32_t W,
@@ -56,7 +57,7 @@ __host__ __device__ inline View make_view(const uint8_t *src, uint8_t *dst, uint
     v.Q = W / 4u;
     v.R = v.Q ? (uint32_t)((N + v.Q - 1) / v.Q) : 0u;
     v.L_last = v.R ? (uint32_t)(N - (uint64_t)(v.R - 1) * v.Q) : 0u;
-    v.pad = 0;
+    v.kmul = 4u;
     return v;
 }
 
@@ -71,527 +72,590 @@ __device__ __forceinline__ uint32_t quarter(uint32_t col, uint32_t L)
     return (col >= L) + (col >= 2 * L) + (col >= 3 * L);
 }
 
-// Byte B (compile-time) of a unit of CH vectors, as a reference to its word.
-template <int CH, int B>
-__device__ __forceinline__ uint32_t &unit_word(uint4 (&o)[CH])
-{
-    uint4 &v = o[B >> 4];
-    constexpr int W = (B >> 2) & 3;
-    return W == 0 ? v.x : W == 1 ? v.y : W == 2 ? v.z : v.w;
-}
-
-template <int CH, int B>
-__device__ __forceinline__ uint32_t unit_word_c(const uint4 (&c)[CH])
-{
-    const uint4 &v = c[B >> 4];
-    constexpr int W = (B >> 2) & 3;
-    return W == 0 ? v.x : W == 1 ? v.y : W == 2 ? v.z : v.w;
-}
-
-// Compile-time plan of the byte moves between a unit's words and its pair
-// words (pair t in byte t%4 of pair word t/4; pixel t's plane byte is unit
-// byte t*CH + PLANE).
-struct UnitPlan {
-    int CH, PLANE;
-    // pixel whose plane byte is unit byte b, or -1
-    __host__ __device__ constexpr int pixel_at(int b) const
-    {
-        return (b >= PLANE && (b - PLANE) % CH == 0 && (b - PLANE) / CH < 16) ? (b - PLANE) / CH
-                                                                             : -1;
-    }
-    // unit word WD: mask of its plane pairs, and the first and last pair
-    // words it takes pairs from
-    __host__ __device__ constexpr uint32_t put_mask(int WD) const
-    {
-        uint32_t m = 0;
-        for (int b = 0; b < 4; ++b)
-            if (pixel_at(4 * WD + b) >= 0)
-                m |= 3u << (8 * b);
-        return m;
-    }
-    __host__ __device__ constexpr int put_qa(int WD) const
-    {
-        for (int b = 0; b < 4; ++b)
-            if (pixel_at(4 * WD + b) >= 0)
-                return pixel_at(4 * WD + b) >> 2;
-        return 0;
-    }
-    __host__ __device__ constexpr int put_qb(int WD) const
-    {
-        for (int b = 3; b >= 0; --b)
-            if (pixel_at(4 * WD + b) >= 0)
-                return pixel_at(4 * WD + b) >> 2;
-        return 0;
-    }
-    // byte_perm selector placing the pairs of unit word WD from pair words
-    // qa (selector 0-3) and qb (4-7); other bytes are masked off later
-    __host__ __device__ constexpr uint32_t put_sel(int WD) const
-    {
-        uint32_t s = 0;
-        for (int b = 0; b < 4; ++b) {
-            const int t = pixel_at(4 * WD + b);
-            const uint32_t d = t < 0 ? 0u : (uint32_t)((t >> 2) == put_qa(WD) ? (t & 3) : 4 + (t & 3));
-            s |= d << (4 * b);
-        }
-        return s;
-    }
-    // pair word Q, byte J: the unit word and byte holding pixel 4Q+J
-    __host__ __device__ constexpr int src_word(int Q, int J) const { return ((4 * Q + J) * CH + PLANE) >> 2; }
-    __host__ __device__ constexpr int src_byte(int Q, int J) const { return ((4 * Q + J) * CH + PLANE) & 3; }
-    // the k-th distinct unit word pair word Q reads (k = 0..3), or -1
-    __host__ __device__ constexpr int gather_src(int Q, int k) const
-    {
-        int n = 0;
-        for (int j = 0; j < 4; ++j) {
-            if (j > 0 && src_word(Q, j) == src_word(Q, j - 1))
-                continue;
-            if (n == k)
-                return src_word(Q, j);
-            ++n;
-        }
-        return -1;
-    }
-    // selector of the first gather step (distinct words 0 and 1) and of the
-    // step adding distinct word k >= 2 to what is gathered so far
-    __host__ __device__ constexpr uint32_t gather_sel0(int Q) const
-    {
-        uint32_t s = 0;
-        const int w0 = gather_src(Q, 0), w1 = gather_src(Q, 1);
-        for (int j = 0; j < 4; ++j) {
-            const int w = src_word(Q, j);
-            const uint32_t d = w == w0 ? (uint32_t)src_byte(Q, j)
-                                       : (w == w1 ? 4u + src_byte(Q, j) : 0u);
-            s |= d << (4 * j);
-        }
-        return s;
-    }
-    __host__ __device__ constexpr uint32_t gather_selk(int Q, int k) const
-    {
-        uint32_t s = 0;
-        const int wk = gather_src(Q, k);
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t d = src_word(Q, j) == wk ? 4u + src_byte(Q, j) : (uint32_t)j;
-            s |= d << (4 * j);
-        }
-        return s;
-    }
+// Where the plane bytes of a unit sit, as byte_perm selectors and masks: a unit's
+// bytes are held as words w[0 .. 4*CH), its 16 plane bytes gathered into (or
+// pairs taken from) four words, byte t%4 of word t/4 for pixel t.  With one
+// channel they are the words themselves; with three, four pixels' plane bytes
+// are bytes ph, ph + 3, ph + 6 and ph + 9 of three words; with four, byte ph of
+// each word.  Selectors made once per launch (or cover) cost one byte_perm in
+// twelve words more than compile-time positions, and one kernel serves every
+// plane and every alignment of it.
+struct PlaneSel {
+    uint32_t get0, get1;         // gather: words 0 and 1, then word 2
+    uint32_t put0, put1, put2;   // three channels: pairs into words 0, 1, 2
+    uint32_t mask0, mask1, mask2;
 };
 
-// Pairs P (pair t in the low two bits of byte t%4 of P[t/4]; the other
-// bits are ignored) into the plane bytes of a unit: per unit word one
-// byte_perm from at most two pair words and one masked merge.
-template <int CH, int PLANE, int WD = 0>
-__device__ __forceinline__ void put_unit(uint4 (&o)[CH], const uint32_t (&P)[4])
+__host__ __device__ inline PlaneSel make_sel(uint32_t ch, uint32_t ph)
 {
-    if constexpr (WD < 4 * CH) {
-        constexpr UnitPlan pl{CH, PLANE};
-        constexpr uint32_t M = pl.put_mask(WD);
-        if constexpr (M != 0) {
-            constexpr int QA = pl.put_qa(WD), QB = pl.put_qb(WD);
-            constexpr uint32_t SEL = pl.put_sel(WD);
-            uint32_t &w = unit_word<CH, 4 * WD>(o);
-            const uint32_t p = __byte_perm(P[QA], P[QB], SEL);
-            w = (w & ~M) | (p & M);
-        }
-        put_unit<CH, PLANE, WD + 1>(o, P);
+    PlaneSel s{};
+    if (ch == 3) {
+        s.get0 = ph == 0 ? 0x0630u : ph == 1 ? 0x0741u : 0x0052u;
+        s.get1 = ph == 0 ? 0x5210u : ph == 1 ? 0x6210u : 0x7410u;
+        s.put0 = ph == 0 ? 0x1440u : ph == 1 ? 0x4404u : 0x4044u;
+        s.put1 = ph == 0 ? 0x4244u : ph == 1 ? 0x2441u : 0x4414u;
+        s.put2 = ph == 0 ? 0x4434u : ph == 1 ? 0x4344u : 0x3442u;
+        s.mask0 = ph == 0 ? 0x03000003u : ph == 1 ? 0x00000300u : 0x00030000u;
+        s.mask1 = ph == 0 ? 0x00030000u : ph == 1 ? 0x03000003u : 0x00000300u;
+        s.mask2 = ph == 0 ? 0x00000300u : ph == 1 ? 0x00030000u : 0x03000003u;
+    } else if (ch == 4) {
+        s.get0 = ph | ((4u + ph) << 4);
+        s.mask0 = 3u << (8 * ph);
+    }
+    return s;
+}
+
+// The 16 plane bytes of a unit.
+template <int CH>
+__device__ __forceinline__ void get_unit(const uint32_t (&w)[4 * CH], const PlaneSel &s,
+                                         uint32_t (&G)[4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if constexpr (CH == 1)
+            G[q] = w[q];
+        else if constexpr (CH == 3)
+            G[q] = __byte_perm(__byte_perm(w[3 * q], w[3 * q + 1], s.get0), w[3 * q + 2], s.get1);
+        else
+            G[q] = __byte_perm(__byte_perm(w[4 * q], w[4 * q + 1], s.get0),
+                               __byte_perm(w[4 * q + 2], w[4 * q + 3], s.get0), 0x5410u);
     }
 }
 
-// Plane bytes of pixels 4Q..4Q+3 of a unit as one word (byte j = pixel
-// 4Q+j's whole plane byte): a chain of byte_perms over the unit words that
-// hold them.
-template <int CH, int PLANE, int Q>
-__device__ __forceinline__ uint32_t gather_word(const uint4 (&c)[CH])
+// Pairs P (the low two bits of each byte; the others are ignored) into the
+// plane bytes of a unit: per word one byte_perm and one masked merge.
+template <int CH>
+__device__ __forceinline__ void put_unit(uint32_t (&w)[4 * CH], const PlaneSel &s,
+                                         const uint32_t (&P)[4])
 {
-    constexpr UnitPlan pl{CH, PLANE};
-    constexpr int W0 = pl.gather_src(Q, 0), W1 = pl.gather_src(Q, 1);
-    constexpr int W2 = pl.gather_src(Q, 2), W3 = pl.gather_src(Q, 3);
-    uint32_t g = __byte_perm(unit_word_c<CH, 4 * W0>(c),
-                             unit_word_c<CH, 4 * (W1 < 0 ? W0 : W1)>(c), pl.gather_sel0(Q));
-    if constexpr (W2 >= 0)
-        g = __byte_perm(g, unit_word_c<CH, 4 * W2>(c), pl.gather_selk(Q, 2));
-    if constexpr (W3 >= 0)
-        g = __byte_perm(g, unit_word_c<CH, 4 * W3>(c), pl.gather_selk(Q, 3));
-    return g;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if constexpr (CH == 1) {
+            w[q] = (w[q] & ~0x03030303u) | (P[q] & 0x03030303u);
+        } else if constexpr (CH == 3) {
+            w[3 * q] = (w[3 * q] & ~s.mask0) | (__byte_perm(P[q], 0u, s.put0) & s.mask0);
+            w[3 * q + 1] = (w[3 * q + 1] & ~s.mask1) | (__byte_perm(P[q], 0u, s.put1) & s.mask1);
+            w[3 * q + 2] = (w[3 * q + 2] & ~s.mask2) | (__byte_perm(P[q], 0u, s.put2) & s.mask2);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                w[4 * q + t] = (w[4 * q + t] & ~s.mask0) |
+                               (__byte_perm(P[q], 0u, 0x1111u * t) & s.mask0);
+        }
+    }
 }
 
-// Plane bytes of a unit's 16 pixels as four words (byte t%4 of G[t/4] =
-// pixel t's plane byte).
-template <int CH, int PLANE>
-__device__ __forceinline__ void get_unit(const uint4 (&c)[CH], uint32_t (&G)[4])
+// 16-byte vectors' words v -> the 16*CH bytes that start d bytes into them (d
+// < 16): the word offset d / 4 by a switch, which a warp takes together where
+// its lanes share d, the byte offset by one byte_perm per word.
+template <int CH, int QW>
+__device__ __forceinline__ void join_words(const uint32_t (&v)[4 * CH + 4], uint32_t sel,
+                                           uint32_t (&o)[4 * CH])
 {
-    if constexpr (CH == 1) {
-        G[0] = c[0].x;
-        G[1] = c[0].y;
-        G[2] = c[0].z;
-        G[3] = c[0].w;
+#pragma unroll
+    for (int q = 0; q < 4 * CH; ++q)
+        o[q] = __byte_perm(v[q + QW], v[q + QW + 1], sel);
+}
+
+template <int CH>
+__device__ __forceinline__ void join_unit(const uint32_t (&v)[4 * CH + 4], uint32_t d,
+                                          uint32_t (&o)[4 * CH])
+{
+    const uint32_t sel = 0x3210u + 0x1111u * (d & 3u);
+    switch (d >> 2) {
+    case 0: join_words<CH, 0>(v, sel, o); break;
+    case 1: join_words<CH, 1>(v, sel, o); break;
+    case 2: join_words<CH, 2>(v, sel, o); break;
+    default: join_words<CH, 3>(v, sel, o); break;
+    }
+}
+
+// Words 4q .. 4q + 3 of w from a vector, and back.
+template <int N>
+__device__ __forceinline__ void set_vec(uint32_t (&w)[N], int q, const uint4 &v)
+{
+    w[4 * q] = v.x;
+    w[4 * q + 1] = v.y;
+    w[4 * q + 2] = v.z;
+    w[4 * q + 3] = v.w;
+}
+
+template <int N>
+__device__ __forceinline__ uint4 get_vec(const uint32_t (&w)[N], int q)
+{
+    return make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+}
+
+// How an image's bytes fall into units.  Units are counted from stego byte h
+// on, a 128-byte boundary of the stego (16-byte in a small image) from which
+// the cover's bytes can be read as whole vectors: unit k is stego bytes [h +
+// 16*CH*k, h + 16*CH*(k + 1)).  As 16*CH bytes are 16 pixels, its plane bytes
+// sit at unit bytes ph + t*CH, t = 0..15, for every k, and belong to pixels x0 +
+// 16k + t: rows of any length and buffers at any address take the same byte
+// positions.  A warp's vectors then start on a cache line: from a 16-byte
+// boundary alone every warp writes two half sectors (8192x8192x3 in place:
+// 87 us against 60).  The unit's cover bytes start d = (cover + h) mod 16
+// bytes into an aligned vector.  The bytes before and after the units (fewer
+// than 400 and 32*CH) are done one by one.
+struct Flat {
+    uint32_t h, d, ph, x0;
+    uint32_t nunits;
+    PlaneSel sel;
+};
+
+// The flat units of a cover; false when it holds none, has too many for 32-bit
+// unit indices (a grid stride of headroom kept) or another channel count.
+// `lead`: with three channels, h moved on by one or two boundaries so that ph =
+// 0, for the kernels that take that position at compile time.
+__host__ __device__ inline bool make_flat(const uint8_t *cover, const uint8_t *stego, uint64_t C,
+                                          uint32_t ch, uint32_t plane, bool lead, Flat &f)
+{
+    if (!(ch == 1 || ch == 3 || ch == 4))
+        return false;
+    const uint32_t align = C >= 16384u ? 128u : 16u;
+    f.h = (uint32_t)(-(uintptr_t)stego & (align - 1u));
+    f.d = (uint32_t)(((uintptr_t)cover + f.h) & 15u);
+    if (f.h < f.d)
+        f.h += align; // the vector around the first cover byte would start before the cover
+    while (lead && ch == 3u && f.h % 3u != plane)
+        f.h += align;
+    f.ph = (plane + 192u * ch - f.h % (3u * ch)) % ch;
+    f.x0 = (f.h + f.ph - plane) / ch;
+    f.nunits = 0;
+    f.sel = make_sel(ch, f.ph);
+    const uint64_t ub = 16u * ch;
+    // one vector more than the units' own is read when d != 0
+    const uint64_t need = f.h + (f.d ? 16u - f.d : 0u);
+    if (C < need + ub)
+        return false;
+    const uint64_t n = (C - need) / ub;
+    if (n >= (1ull << 31))
+        return false;
+    f.nunits = (uint32_t)n;
+    return true;
+}
+
+// Quotient of a pixel or run index by a row length: in 32 bits where it fits
+// (a 64-bit division is some 100 instructions, a microsecond of a small
+// launch).
+__device__ __forceinline__ uint32_t row_of(uint64_t x, uint32_t W)
+{
+    return (x >> 32) == 0 ? (uint32_t)x / W : (uint32_t)(x / W);
+}
+
+// Units with carrying pixels: a prefix of the image's units.
+__device__ __forceinline__ uint32_t carrying_units(const View &a, const Flat &f)
+{
+    const uint64_t last = a.R ? (uint64_t)(a.R - 1) * a.W + 4ull * a.L_last : 0ull; // pixels before its end
+    const uint64_t n = last > f.x0 ? (last - f.x0 + 15u) / 16u : 0ull;
+    return (uint32_t)(n < f.nunits ? n : f.nunits);
+}
+
+// (row, column) advanced by dr rows and dc < W columns.
+__device__ __forceinline__ void rc_add(uint32_t &r, uint32_t &c, uint32_t dr, uint32_t dc,
+                                       uint32_t W)
+{
+    r += dr;
+    if (c >= W - dc) {
+        c -= W - dc;
+        ++r;
     } else {
-        G[0] = gather_word<CH, PLANE, 0>(c);
-        G[1] = gather_word<CH, PLANE, 1>(c);
-        G[2] = gather_word<CH, PLANE, 2>(c);
-        G[3] = gather_word<CH, PLANE, 3>(c);
+        c += dc;
     }
 }
 
-// Pairs of a unit's plane bytes (their low two bits) into a SWAR pair array
-// (pair t in byte t%4 of P[t/4]; P starts zeroed), one shift and mask per
-// pixel: in the extraction this measured faster than the byte_perm gather.
-template <int CH, int PLANE, int T = 0>
-__device__ __forceinline__ void get_pairs(const uint4 (&c)[CH], uint32_t (&P)[4])
+// Message bytes off .. off + 15 one by one, 0 outside the message, four loads
+// in flight together (a loop, to keep the code of this rare case small).
+__device__ __forceinline__ void window_bytes(const uint8_t *__restrict__ msg, uint64_t N,
+                                             int64_t off, uint32_t (&m)[4])
 {
-    if constexpr (T < 16) {
-        constexpr int B = T * CH + PLANE, S = 8 * (B & 3);
-        const uint32_t w = unit_word_c<CH, B & ~3>(c);
-        P[T >> 2] |= ((w >> S) & 3u) << (8 * (T & 3));
-        get_pairs<CH, PLANE, T + 1>(c, P);
+    m[0] = m[1] = m[2] = m[3] = 0u;
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q, off += 4) {
+        uint32_t b[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            b[t] = (uint64_t)(off + t) < N ? (uint32_t)__ldg(msg + (off + t)) : 0u;
+        m[0] = m[1];
+        m[1] = m[2];
+        m[2] = m[3];
+        m[3] = __byte_perm(__byte_perm(b[0], b[1], 0x0040u), __byte_perm(b[2], b[3], 0x0040u), 0x5410u);
     }
 }
 
-// Per-pixel path for a unit that crosses a quarter boundary or the end of
-// the carrying columns: pixel T at column colf + T.
-template <int CH, int PLANE, int T>
-__device__ __forceinline__ void slow_unit(uint4 (&o)[CH], uint32_t colf, uint32_t L,
-                                          const uint8_t *__restrict__ mrow)
+// Message bytes off .. off + 15 as four words: one vector load where they lie
+// on a 16-byte boundary, else the five aligned words around them and a funnel
+// shift each (rows of W pixels start at any message address when floor(W/4) is
+// not a multiple of 4; byte loads took 16 instructions and requests), else,
+// where those words are not all inside the message, one by one.
+__device__ __forceinline__ void load_window(const uint8_t *__restrict__ msg, uint64_t N,
+                                            int64_t off, uint32_t (&m)[4])
 {
-    if constexpr (T < 16) {
-        const uint32_t col = colf + T;
-        if (col < 4 * L) {
-            const uint32_t i = quarter(col, L);
-            const uint32_t p = (__ldg(mrow + (col - i * L)) >> (2 * i)) & 3u;
-            constexpr int B = T * CH + PLANE, S = 8 * (B & 3);
-            uint32_t &w = unit_word<CH, B>(o);
-            w = (w & ~(3u << S)) | (p << S);
-        }
-        slow_unit<CH, PLANE, T + 1>(o, colf, L, mrow);
-    }
-}
-
-// Four 32-bit words of message bytes mp[0..15] (mp 4-byte aligned or not).
-__device__ __forceinline__ void load16(const uint8_t *__restrict__ mp, uint32_t (&m)[4])
-{
-    if (((uintptr_t)mp & 15u) == 0) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(mp));
+    const uintptr_t p = (uintptr_t)msg + (uintptr_t)off;
+    const uint32_t s = (uint32_t)(p & 3u);
+    const uintptr_t w0 = p - s;
+    if (off >= 0 && (p & 15u) == 0 && (uint64_t)off + 16u <= N) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
         m[0] = v.x;
         m[1] = v.y;
         m[2] = v.z;
         m[3] = v.w;
-    } else if (((uintptr_t)mp & 3u) == 0) {
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(mp);
+    } else if (off >= (int64_t)s && (uint64_t)(off - s) + 20u <= N) {
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(w0);
+        uint32_t v[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            v[q] = __ldg(w + q);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            m[q] = __ldg(w + q);
+            m[q] = __funnelshift_r(v[q], v[q + 1], 8u * s);
     } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            m[q] = (uint32_t)__ldg(mp + 4 * q) | ((uint32_t)__ldg(mp + 4 * q + 1) << 8) |
-                   ((uint32_t)__ldg(mp + 4 * q + 2) << 16) | ((uint32_t)__ldg(mp + 4 * q + 3) << 24);
+        window_bytes(msg, N, off, m);
     }
 }
 
-// Changed plane bytes and squared error of a unit from its new and old
-// plane bytes (byte t%4 of word t/4 = pixel t; only the low two bits can
-// differ, the other bits are ignored), added to 32-bit per-unit counts.
-__device__ __forceinline__ void plane_stats(const uint32_t (&Gn)[4], const uint32_t (&Go)[4],
-                                            uint32_t &n, uint32_t &s)
+// Bytes [t, e) of 16 (byte t%4 of word t/4) as a mask of word q.
+__device__ __forceinline__ uint32_t span_mask(uint32_t t, uint32_t e, int q)
+{
+    const int lo = (int)t - 4 * q, hi = (int)e - 4 * q;
+    const uint32_t a = lo <= 0 ? 0xFFFFFFFFu : lo >= 4 ? 0u : 0xFFFFFFFFu << (8 * lo);
+    const uint32_t b = hi >= 4 ? 0xFFFFFFFFu : hi <= 0 ? 0u : 0xFFFFFFFFu >> (32 - 8 * hi);
+    return a & b;
+}
+
+// G[q] takes the low two bits of m[q] >> sh under the byte mask of [t, e).
+__device__ __forceinline__ void merge_pairs(uint32_t (&G)[4], const uint32_t (&m)[4], uint32_t sh,
+                                            uint32_t t, uint32_t e)
 {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const uint32_t d = __vabsdiffu4(Gn[q] & 0x03030303u, Go[q] & 0x03030303u);
-        n += __popc((d | (d >> 1)) & 0x01010101u);
-        s = __dp4a(d, d, s);
+        const uint32_t k = span_mask(t, e, q);
+        G[q] = (G[q] & ~k) | ((m[q] >> sh) & k);
     }
 }
 
-// (row, unit column) advanced by dr rows and dc < upr units.
-__device__ __forceinline__ void rc_add(uint32_t &r, uint32_t &c, uint32_t dr, uint32_t dc,
-                                       uint32_t upr)
+// The pairs of 16 pixels that start at (r, col) and do not all lie in one
+// quarter of a row; G holds the pixels' plane bytes, whose low two bits the
+// pixels that carry nothing keep.  Between full rows of quarters of at least
+// 16 pixels there are two spans, the pixels before the end of the quarter and
+// those of the next quarter (or, past the at most three columns that carry
+// nothing, of the next row), one message window and one masked merge each;
+// otherwise quarter by quarter.  At a row length of 5471 one unit in 68 comes
+// here, at 1000 one in 12, so that nearly every warp there has one (gray
+// 5471x3647: 15.1 us, with the loop alone 16.9).
+__device__ __forceinline__ void edge_pairs(const View &a, uint32_t r, uint32_t col,
+                                           uint32_t (&G)[4])
 {
-    r += dr;
-    c += dc;
-    if (c >= upr) {
-        c -= upr;
-        ++r;
-    }
-}
-
-// Units with carrying pixels, a prefix of the image's units: every unit of
-// rows 0..R-2 (4Q = W when W is a multiple of 16) and the first
-// ceil(L_last/4) of row R-1.
-__device__ __forceinline__ uint32_t carrying_units(const View &a, uint32_t upr)
-{
-    return a.R ? (a.R - 1) * upr + (a.L_last + 3) / 4 : 0u;
-}
-
-constexpr int kStageWarps = 8; // units_embed_async runs in CTAs of at most 256 threads
-
-// One pass over units k = k_first + i*step (+ u*blockDim.x, u < UT),
-// k < k_end, of an image whose rows are whole units and whose buffers are
-// 16-byte aligned, each thread on its own units: every load of an iteration
-// (cover, then message) is issued before any arithmetic.  With one channel
-// the lanes' single-vector units are consecutive (coalesced); with three or
-// four a lane's unit lies 16*CH bytes from its neighbour's, which
-// units_embed_async avoids and the batched kernels accept for their register
-// budget.  Out of place every unit is written (units without carrying pixels
-// are copied); in place (INPLACE) k_end is cut to the carrying units, each
-// unit read and written back by the same thread.
-template <int CH, int PLANE, bool STATS, int UT, bool INPLACE = false>
-__device__ __forceinline__ void units_embed(const View &a, uint32_t k_first, uint32_t k_end,
-                                            uint32_t step, unsigned long long &changed,
-                                            unsigned long long &sse)
-{
-    const uint32_t upr = a.W / 16; // units per row
-    if (upr == 0)
+    uint32_t m[4];
+    if (a.Q >= 16u && r + 2 < a.R) {
+        const uint32_t i = quarter(col, a.Q);
+        const bool carries = col < 4u * a.Q;
+        const uint32_t n = carries && (i + 1) * a.Q - col < 16u ? (i + 1) * a.Q - col : 0u;
+        const uint64_t row = (uint64_t)r * a.Q;
+        if (n) { // the first span
+            load_window(a.msg_in, a.N, (int64_t)(row + col - i * a.Q), m);
+            merge_pairs(G, m, 2 * i, 0, n);
+        }
+        // the second: byte 0 of the next quarter, or of the next row
+        const bool same = i < 3u;
+        const uint32_t t = same ? n : a.W - col;
+        load_window(a.msg_in, a.N, (int64_t)(same ? row : row + a.Q) - (int64_t)t, m);
+        merge_pairs(G, m, same ? 2 * i + 2 : 0u, t, 16u);
         return;
-    const uint32_t carry = carrying_units(a, upr);
+    }
+    uint32_t t = 0;
+#pragma unroll 1
+    while (t < 16 && r < a.R) {
+        const uint32_t L = row_len(a, r), i = quarter(col, L);
+        if (col < 4u * L) { // L >= 1 for r < R
+            const uint32_t left = (i + 1) * L - col, n = left < 16u - t ? left : 16u - t;
+            load_window(a.msg_in, a.N, (int64_t)((uint64_t)r * a.Q + (col - i * L)) - (int64_t)t, m);
+            merge_pairs(G, m, 2 * i, t, t + n);
+            t += n;
+            col += n;
+        }
+        if (col >= 4u * L) { // the columns past the last quarter carry nothing
+            const uint32_t rest = a.W - col;
+            t = rest < 16u ? t + rest : 16u;
+            col = 0;
+            ++r;
+        }
+    }
+}
+
+// What one unit needs besides its cover vectors: how it is embedded (mode 0
+// copy only, 1 all 16 pixels in one quarter of a row, 2 otherwise), its first
+// pixel (mode 2) and, in mode 1, its shift and 16 message bytes.
+struct UnitJob {
+    uint32_t mode, r, col, sh;
+    uint32_t m[4];
+};
+
+__device__ __forceinline__ void plan_unit(const View &a, bool carries, uint32_t r, uint32_t col,
+                                          UnitJob &J)
+{
+    J.mode = 0;
+    if (carries) {
+        const uint32_t L = row_len(a, r), i = quarter(col, L), e = (i + 1) * L;
+        if (col < e && e - col >= 16u) {
+            J.mode = 1;
+            J.sh = 2 * i;
+            load_window(a.msg_in, a.N, (int64_t)((uint64_t)r * a.Q + (col - i * L)), J.m);
+        } else {
+            J.mode = 2;
+            J.r = r;
+            J.col = col;
+        }
+    }
+}
+
+// Embeds a planned unit in registers (mode != 0).
+template <int CH, bool STATS>
+__device__ __forceinline__ void embed_unit(const View &a, const UnitJob &J, const PlaneSel &sel,
+                                           uint32_t (&o)[4 * CH], unsigned long long &changed,
+                                           unsigned long long &sse)
+{
+    uint32_t Gn[4], Go[4];
+    if (STATS || J.mode == 2)
+        get_unit<CH>(o, sel, Go); // old plane bytes
+    if (J.mode == 1) {
+        // pair of the unit's quarter in the low two bits of each byte
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            Gn[q] = J.m[q] >> J.sh;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            Gn[q] = Go[q];
+        edge_pairs(a, J.r, J.col, Gn);
+    }
+    put_unit<CH>(o, sel, Gn);
+    if (STATS) {
+        uint32_t d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            d[q] = (Gn[q] ^ Go[q]) & 0x03030303u;
+        unit_stats<2>(Gn, Go, d, a.kmul, changed, sse);
+    }
+}
+
+// The bytes outside the units, [0, f.h) and [f.h + 16*CH*nunits, C), one per
+// thread of the calling CTA; `head` and `tail` choose which.  In place only
+// those that change are written.
+template <bool STATS>
+__device__ __forceinline__ void edge_bytes(const View &a, const Flat &f, bool head, bool tail,
+                                           unsigned long long &changed, unsigned long long &sse)
+{
+    const uint64_t C = (uint64_t)a.W * a.H * a.channels;
+    const uint64_t t0 = f.h + 16ull * a.channels * f.nunits;
+    const uint32_t nh = head ? f.h : 0u, nt = tail ? (uint32_t)(C - t0) : 0u;
+    for (uint32_t e = threadIdx.x; e < nh + nt; e += blockDim.x) {
+        const uint64_t k = e < nh ? e : t0 + (e - nh);
+        const uint64_t x = a.channels == 1 ? k : a.channels == 4 ? k >> 2 : k / 3u;
+        const uint32_t cb = a.src[k];
+        uint32_t ob = cb;
+        if ((uint32_t)(k - x * a.channels) == a.plane) {
+            const uint32_t r = row_of(x, a.W);
+            const uint32_t col = (uint32_t)(x - (uint64_t)r * a.W);
+            const uint32_t L = r < a.R ? row_len(a, r) : 0u;
+            if (col < 4u * L) {
+                const uint32_t i = quarter(col, L);
+                ob = (cb & 0xFCu) | ((__ldg(a.msg_in + (uint64_t)r * a.Q + (col - i * L)) >> (2 * i)) & 3u);
+            }
+        }
+        if (ob != cb || a.dst != a.src)
+            a.dst[k] = (uint8_t)ob;
+        if (STATS) {
+            const uint32_t d = ob > cb ? ob - cb : cb - ob;
+            changed += d != 0;
+            sse += d * d;
+        }
+    }
+}
+
+// Shared memory of a units_embed_async CTA of at most 256 threads: two stages
+// of a warp's vectors, and the one after them.
+constexpr int kStageWarps = 8;
+template <int CH>
+__host__ __device__ constexpr uint32_t stage_vectors()
+{
+    return kStageWarps * 2 * (unit_stage_slots<CH>() + 1);
+}
+
+// One pass over units k = k_first + i*step (+ u*blockDim.x, u < UT), k <
+// k_end, each thread on its own units: every load of an iteration (cover,
+// then message) is issued before any arithmetic.  With one channel the lanes'
+// single-vector units are consecutive (coalesced); with three or four a lane's
+// unit lies 16*CH bytes from its neighbour's, which units_embed_async avoids
+// and the batched kernels accept for their register budget.  Cover and stego
+// at different addresses mod 16: the vector after the unit's own is loaded too
+// (the neighbour's first: an L1 hit) and the bytes joined.  Out of place every
+// unit is written (units without carrying pixels are copied); in place
+// (INPLACE) k_end is cut to the carrying units, each unit read and written
+// back by the same thread.
+template <int CH, bool STATS, int UT, bool INPLACE = false, bool LEAD = false>
+__device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32_t k_first,
+                                            uint32_t k_end, uint32_t step,
+                                            unsigned long long &changed, unsigned long long &sse)
+{
+    const uint32_t carry = carrying_units(a, f);
     if (INPLACE && k_end > carry)
         k_end = carry;
-    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.dst);
-    // row and unit column of the thread's unit: with several units per thread
-    // kept by additions (the strides blockDim.x and step in whole rows and
-    // remaining units), with one unit divided out (fewer live registers)
-    constexpr bool TRACK = UT > 1;
-    uint32_t r0 = 0, u0 = 0, tr = 0, tc = 0, sr = 0, sc = 0;
-    if constexpr (TRACK) {
-        r0 = k_first / upr;
-        u0 = k_first - r0 * upr;
-        tr = blockDim.x / upr;
-        tc = blockDim.x - tr * upr;
-        sr = step / upr;
-        sc = step - sr * upr;
-    }
+    if (k_first >= k_end)
+        return;
+    const PlaneSel sel = LEAD && CH == 3 ? make_sel(3, 0) : f.sel;
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src + f.h - f.d);
+    uint4 *dst = reinterpret_cast<uint4 *>(a.dst + f.h);
+    // row and column of the thread's first pixel, kept by additions
+    const uint64_t x = f.x0 + 16ull * k_first;
+    uint32_t r0 = row_of(x, a.W), c0 = (uint32_t)(x - (uint64_t)r0 * a.W);
+    const uint32_t tr = UT > 1 ? 16u * blockDim.x / a.W : 0u;
+    const uint32_t tc = UT > 1 ? 16u * blockDim.x - tr * a.W : 0u;
+    const uint32_t sr = 16u * step / a.W, sc = 16u * step - sr * a.W; // 16 * step < 2^32
     for (uint32_t k0 = k_first; k0 < k_end; k0 += step) {
-        uint4 c[UT][CH];
+        uint32_t c[UT][4 * CH + 4];
 #pragma unroll
         for (int u = 0; u < UT; ++u) {
             const uint32_t k = k0 + u * blockDim.x;
             if (k < k_end) {
 #pragma unroll
                 for (int q = 0; q < CH; ++q)
-                    c[u][q] = __ldcs(src + (uint64_t)k * CH + q);
+                    set_vec(c[u], q, __ldcs(src + (uint64_t)k * CH + q));
+                if (!INPLACE && f.d)
+                    set_vec(c[u], CH, __ldcs(src + (uint64_t)k * CH + CH));
             }
         }
-        int mode[UT]; // 0: copy only, 1: one quarter (SWAR), 2: per pixel
-        uint32_t colf[UT], L[UT], i0[UT], m[UT][4];
-        const uint8_t *mrow[UT];
-        uint32_t r = r0, uc = u0;
+        UnitJob J[UT];
+        uint32_t r = r0, col = c0;
 #pragma unroll
         for (int u = 0; u < UT; ++u) {
             const uint32_t k = k0 + u * blockDim.x;
-            if constexpr (TRACK) {
-                if (u > 0)
-                    rc_add(r, uc, tr, tc, upr);
-            } else {
-                r = k / upr;
-                uc = k - r * upr;
-            }
-            mode[u] = 0;
-            if (k < k_end && k < carry) {
-                colf[u] = 16u * uc;
-                L[u] = row_len(a, r);
-                mrow[u] = a.msg_in + (uint64_t)r * a.Q;
-                i0[u] = quarter(colf[u], L[u]);
-                if (colf[u] + 15 < 4 * L[u] && quarter(colf[u] + 15, L[u]) == i0[u]) {
-                    mode[u] = 1;
-                    load16(mrow[u] + (colf[u] - i0[u] * L[u]), m[u]);
-                } else {
-                    mode[u] = 2;
-                }
-            }
+            if (u > 0)
+                rc_add(r, col, tr, tc, a.W);
+            plan_unit(a, k < k_end && k < carry, r, col, J[u]);
         }
 #pragma unroll
         for (int u = 0; u < UT; ++u) {
             const uint32_t k = k0 + u * blockDim.x;
             if (k >= k_end)
                 continue;
-            uint4(&o)[CH] = c[u]; // rewritten in registers
-            uint32_t Gn[4], Go[4];
-            if (STATS && mode[u])
-                get_unit<CH, PLANE>(o, Go); // old plane bytes
-            if (mode[u] == 1) {
-                // pair of quarter i0 in the low two bits of each byte
+            uint32_t o[4 * CH];
+            if (!INPLACE && f.d) {
+                join_unit<CH>(c[u], f.d, o);
+            } else {
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    Gn[q] = m[u][q] >> (2 * i0[u]);
-                if constexpr (CH == 1) {
-                    o[0].x = (o[0].x & 0xFCFCFCFCu) | (Gn[0] & 0x03030303u);
-                    o[0].y = (o[0].y & 0xFCFCFCFCu) | (Gn[1] & 0x03030303u);
-                    o[0].z = (o[0].z & 0xFCFCFCFCu) | (Gn[2] & 0x03030303u);
-                    o[0].w = (o[0].w & 0xFCFCFCFCu) | (Gn[3] & 0x03030303u);
-                } else {
-                    put_unit<CH, PLANE>(o, Gn);
-                }
-            } else if (mode[u] == 2) {
-                slow_unit<CH, PLANE, 0>(o, colf[u], L[u], mrow[u]);
-                if (STATS)
-                    get_unit<CH, PLANE>(o, Gn);
+                for (int q = 0; q < 4 * CH; ++q)
+                    o[q] = c[u][q];
             }
-            if (STATS && mode[u]) {
-                uint32_t n = 0, sq = 0; // at most 16 pairs changed, 9 each
-                plane_stats(Gn, Go, n, sq);
-                changed += n;
-                sse += sq;
-            }
+            if (J[u].mode)
+                embed_unit<CH, STATS>(a, J[u], sel, o, changed, sse);
 #pragma unroll
             for (int q = 0; q < CH; ++q)
-                __stcs(dst + (uint64_t)k * CH + q, o[q]);
+                __stcs(dst + (uint64_t)k * CH + q, get_vec(o, q));
         }
-        if constexpr (TRACK)
-            rc_add(r0, u0, sr, sc, upr);
-    }
-}
-
-// What one unit needs besides its cover vectors: how it is embedded (mode
-// 0 copy only, 1 one quarter, 2 per pixel), its column, row length,
-// quarter, message row and, in mode 1, its 16 message bytes.
-struct UnitJob {
-    uint32_t mode, colf, L, i0;
-    const uint8_t *mrow;
-    uint32_t m[4];
-};
-
-__device__ __forceinline__ void plan_unit(const View &a, uint32_t k, uint32_t k_end,
-                                          uint32_t carry, uint32_t r, uint32_t uc, UnitJob &J)
-{
-    J.mode = 0;
-    if (k < k_end && k < carry) {
-        J.colf = 16u * uc;
-        J.L = row_len(a, r);
-        J.mrow = a.msg_in + (uint64_t)r * a.Q;
-        J.i0 = quarter(J.colf, J.L);
-        if (J.colf + 15 < 4 * J.L && quarter(J.colf + 15, J.L) == J.i0) {
-            J.mode = 1;
-            load16(J.mrow + (J.colf - J.i0 * J.L), J.m);
-        } else {
-            J.mode = 2;
-        }
+        rc_add(r0, c0, sr, sc, a.W);
     }
 }
 
 // units_embed for CH > 1 with a two-stage copy pipeline per warp: while the
-// warp embeds the units of one iteration from shared memory, the cover
-// vectors of its next iteration are already on their way there
-// (cp.async, memory order, coalesced) and the next units' message bytes on
-// their way to registers.  Same arguments and results as units_embed; CTAs
-// of at most 256 threads.
-template <int CH, int PLANE, bool STATS, int UT, bool INPLACE = false>
-__device__ __forceinline__ void units_embed_async(const View &a, uint32_t k_first,
+// warp embeds its 32 units from shared memory, the cover vectors of its next
+// 32 are already on their way there (cp.async, memory order, coalesced) and
+// the next units' message bytes on their way to registers.  SHIFTED: cover and
+// stego at different addresses mod 16 (f.d != 0); the stage then holds the
+// 32*CH + 1 aligned cover vectors around the warp's bytes, of which each lane
+// reads CH + 1.  Same results as units_embed; `stage` is the CTA's
+// stage_vectors<CH>() vectors of shared memory.
+template <int CH, bool STATS, bool SHIFTED, bool INPLACE = false>
+__device__ __forceinline__ void units_embed_async(const View &a, const Flat &f, uint32_t k_first,
                                                   uint32_t k_end, uint32_t step,
                                                   unsigned long long &changed,
-                                                  unsigned long long &sse)
+                                                  unsigned long long &sse, uint4 *stage)
 {
     static_assert(CH > 1, "one-channel units are single vectors, loaded coalesced as they are");
-    const uint32_t upr = a.W / 16;
-    if (upr == 0)
-        return;
-    const uint32_t carry = carrying_units(a, upr);
+    const uint32_t carry = carrying_units(a, f);
     if (INPLACE && k_end > carry)
         k_end = carry;
-    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.dst);
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src + f.h - (SHIFTED ? f.d : 0u));
+    uint4 *dst = reinterpret_cast<uint4 *>(a.dst + f.h);
     const uint32_t lane = threadIdx.x & 31u;
-    constexpr uint32_t SV = unit_stage_slots<CH>();
-    constexpr uint32_t WS = 2 * UT * SV; // two stages per warp
-    __shared__ uint4 stage[kStageWarps * WS];
-    uint4 *const sw = stage + (threadIdx.x >> 5) * WS;
+    constexpr uint32_t SV = unit_stage_slots<CH>() + (SHIFTED ? 1u : 0u);
+    uint4 *const sw = stage + (threadIdx.x >> 5) * 2 * SV;
     const uint64_t vend = (uint64_t)k_end * CH;
-    const uint32_t tr = blockDim.x / upr, tc = blockDim.x - tr * upr;
-    const uint32_t sr = step / upr, sc = step - sr * upr;
-    uint32_t r0 = k_first / upr, u0 = k_first - r0 * upr;
-
-    // the warp's vectors of the iteration at lane 0's unit kb -> stage s
-    auto issue = [&](uint32_t kb, uint32_t s) {
-#pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint64_t v0 = (uint64_t)(kb + u * blockDim.x) * CH;
-#pragma unroll
-            for (int j = 0; j < CH; ++j)
-                if (v0 + 32u * j + lane < vend)
-                    cp_async16(sw + s * UT * SV + u * SV + unit_stage_slot<CH>(32u * j + lane),
-                               src + v0 + 32u * j + lane);
-        }
-        cp_async_commit();
-    };
-    auto plan = [&](uint32_t k0, uint32_t r, uint32_t uc, UnitJob (&J)[UT]) {
-#pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            if (u > 0)
-                rc_add(r, uc, tr, tc, upr);
-            plan_unit(a, k0 + u * blockDim.x, k_end, carry, r, uc, J[u]);
-        }
-    };
-
     uint32_t k0 = k_first; // the lane's first unit; k0 - lane is the same for the warp
     if (k0 - lane >= k_end)
         return;
-    UnitJob J[UT];
+    const uint64_t x = f.x0 + 16ull * k_first;
+    uint32_t r0 = row_of(x, a.W), c0 = (uint32_t)(x - (uint64_t)r0 * a.W);
+    const uint32_t sr = 16u * step / a.W, sc = 16u * step - sr * a.W; // 16 * step < 2^32
+
+    // the warp's vectors from lane 0's unit kb on -> stage s
+    auto issue = [&](uint32_t kb, uint32_t s) {
+        const uint64_t v0 = (uint64_t)kb * CH;
+#pragma unroll
+        for (int j = 0; j < CH; ++j)
+            if (v0 + 32u * j + lane < vend + (SHIFTED ? 1u : 0u))
+                cp_async16(sw + s * SV + unit_stage_slot<CH>(32u * j + lane), src + v0 + 32u * j + lane);
+        if (SHIFTED && lane == 0 && v0 + 32u * CH <= vend)
+            cp_async16(sw + s * SV + unit_stage_slot<CH>(32u * CH), src + v0 + 32u * CH);
+        cp_async_commit();
+    };
+
+    UnitJob J;
     issue(k0 - lane, 0);
-    plan(k0, r0, u0, J);
+    plan_unit(a, k0 < k_end && k0 < carry, r0, c0, J);
     uint32_t s = 0;
     for (;;) {
         const uint32_t kn = k0 + step;
         const bool next = kn - lane < k_end; // kn < 2^32: units and steps stay below 2^31
-        UnitJob Jn[UT];
-        rc_add(r0, u0, sr, sc, upr);
+        UnitJob Jn;
         if (next) {
+            rc_add(r0, c0, sr, sc, a.W);
             issue(kn - lane, s ^ 1u);
-            plan(kn, r0, u0, Jn);
+            plan_unit(a, kn < k_end && kn < carry, r0, c0, Jn);
             cp_async_wait<1>(); // this iteration's copies landed (the next may be pending)
         } else {
             cp_async_wait<0>();
         }
         __syncwarp(); // every lane's copies visible to the warp
-        uint4 *const st = sw + s * UT * SV;
+        uint4 *const st = sw + s * SV;
+        if constexpr (SHIFTED) {
+            uint32_t o[4 * CH];
+            if (k0 < k_end) {
+                uint32_t v[4 * CH + 4];
 #pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint32_t k = k0 + u * blockDim.x;
-            if (k >= k_end)
-                continue;
-            uint4 o[CH];
-#pragma unroll
-            for (int q = 0; q < CH; ++q)
-                o[q] = st[u * SV + unit_stage_slot<CH>(CH * lane + q)];
-            uint32_t Gn[4], Go[4];
-            if (STATS && J[u].mode)
-                get_unit<CH, PLANE>(o, Go);
-            if (J[u].mode == 1) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    Gn[q] = J[u].m[q] >> (2 * J[u].i0);
-                put_unit<CH, PLANE>(o, Gn);
-            } else if (J[u].mode == 2) {
-                slow_unit<CH, PLANE, 0>(o, J[u].colf, J[u].L, J[u].mrow);
-                if (STATS)
-                    get_unit<CH, PLANE>(o, Gn);
+                for (int q = 0; q <= CH; ++q)
+                    set_vec(v, q, st[unit_stage_slot<CH>(CH * lane + q)]);
+                join_unit<CH>(v, f.d, o);
+                if (J.mode)
+                    embed_unit<CH, STATS>(a, J, f.sel, o, changed, sse);
             }
-            if (STATS && J[u].mode) {
-                uint32_t n = 0, sq = 0;
-                plane_stats(Gn, Go, n, sq);
-                changed += n;
-                sse += sq;
-            }
-            if (J[u].mode) {
+            __syncwarp(); // the neighbour has read this lane's first vector
+            if (k0 < k_end) {
 #pragma unroll
                 for (int q = 0; q < CH; ++q)
-                    st[u * SV + unit_stage_slot<CH>(CH * lane + q)] = o[q];
+                    st[unit_stage_slot<CH>(CH * lane + q)] = get_vec(o, q);
             }
+        } else if (k0 < k_end && J.mode) {
+            uint32_t o[4 * CH];
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+                set_vec(o, q, st[unit_stage_slot<CH>(CH * lane + q)]);
+            embed_unit<CH, STATS>(a, J, f.sel, o, changed, sse);
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+                st[unit_stage_slot<CH>(CH * lane + q)] = get_vec(o, q);
         }
         __syncwarp(); // the rewritten units visible to the storing lanes
+        const uint64_t v0 = (uint64_t)(k0 - lane) * CH;
 #pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint64_t v0 = (uint64_t)(k0 - lane + u * blockDim.x) * CH;
-#pragma unroll
-            for (int j = 0; j < CH; ++j)
-                if (v0 + 32u * j + lane < vend)
-                    __stcs(dst + v0 + 32u * j + lane, st[u * SV + unit_stage_slot<CH>(32u * j + lane)]);
-        }
+        for (int j = 0; j < CH; ++j)
+            if (v0 + 32u * j + lane < vend)
+                __stcs(dst + v0 + 32u * j + lane, st[unit_stage_slot<CH>(32u * j + lane)]);
         if (!next)
             break;
-        // stage s is refilled two iterations on, after this lane's reads of
-        // its own memory-order slots above
-#pragma unroll
-        for (int u = 0; u < UT; ++u)
-            J[u] = Jn[u];
+        // stage s is refilled two iterations on, after every lane passed the
+        // barriers above and read its own memory-order slots
+        J = Jn;
         k0 = kn;
         s ^= 1u;
     }
@@ -675,71 +739,216 @@ __device__ __forceinline__ void rows_copy(const View &a, uint32_t r0, uint32_t r
     }
 }
 
-// Extraction over runs k = k_first + i*step < k_end of 16 message bytes of a
-// carrying row (rpr = ceil(Q/16) runs per row): the four units at columns
-// i*L + j0 are read as vectors when every one is a whole 16-byte aligned
-// unit, byte by byte otherwise.
-template <int CH, int PLANE>
-__device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, uint64_t k_end,
-                                             uint64_t step)
+// Runs of an extraction: row r's message bytes lie in at most run_row()
+// 16-byte blocks of the output, counted from the block that holds its first
+// byte; run k is block k mod run_row() of row k / run_row().  A run takes the
+// bytes of its block that are its row's: all 16 but in the row's first and
+// last block, which it shares with the neighbouring rows' runs.
+// Where rows and quarters of the image and rows of the output are whole
+// 16-byte vectors (runs_aligned: W a multiple of 64, both buffers 16-byte
+// aligned), every run of a full row reads aligned vectors and writes one.
+__host__ __device__ inline bool runs_aligned(const View &v)
 {
-    const uint32_t rpr = (a.Q + 15) / 16;
-    for (uint64_t k = k_first; k < k_end; k += step) {
-        const uint32_t r = (uint32_t)(k / rpr);
-        const uint32_t j0 = 16u * (uint32_t)(k - (uint64_t)r * rpr);
-        const uint32_t L = row_len(a, r);
-        if (j0 >= L)
-            continue;
-        const uint64_t prow = (uint64_t)r * a.W;
-        uint8_t *mp = a.msg_out + (uint64_t)r * a.Q + j0;
-        // whole unit per quarter, and every quarter's unit 16-byte aligned:
-        // the first one aligned and the quarter stride L*CH a multiple of 16
-        const bool fast = j0 + 16 <= L && ((uint64_t)L * CH) % 16u == 0 &&
-                          (((uintptr_t)(a.src + (prow + j0) * CH)) & 15u) == 0;
-        if (fast) {
-            uint4 c[4][CH];
+    return v.W % 64u == 0 && (((uintptr_t)v.src | (uintptr_t)v.msg_out) & 15u) == 0;
+}
+
+__host__ __device__ inline uint32_t run_row(const View &v)
+{
+    return runs_aligned(v) ? v.Q / 16u : (uint32_t)(((uint64_t)v.Q + 30u) / 16u);
+}
+
+__host__ __device__ inline uint64_t run_count(const View &v)
+{
+    return v.Q ? (uint64_t)v.R * run_row(v) : 0u;
+}
+
+// Quarter i's plane bytes P into M: pair t in bits 2i of byte t.
+__device__ __forceinline__ void take_pairs(uint32_t (&M)[4], const uint32_t (&P)[4], int i)
+{
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 *u = reinterpret_cast<const uint4 *>(
-                    a.src + (prow + (uint64_t)L * i + j0) * CH);
+    for (int q = 0; q < 4; ++q)
+        M[q] |= (P[q] & 0x03030303u) << (2 * i);
+}
+
+// The pairs of the 16 pixels whose first plane byte is byte `off` of the image,
+// for G quarters from i0 on, `stride` bytes apart.  Each is read as the CH (on a
+// 16-byte boundary) or CH + 1 aligned vectors around its bytes where those lie
+// inside the image, else byte by byte, pixels [t, e) alone.
+template <int CH, int G>
+__device__ __forceinline__ void run_quarters(const View &a, uint64_t C, int64_t off,
+                                             uint64_t stride, int i0, uint32_t t, uint32_t e,
+                                             uint32_t (&M)[4])
+{
+    const uintptr_t lo = (uintptr_t)a.src, hi = lo + C;
+    uint32_t v[G][4 * CH + 4];
+    bool whole[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const uintptr_t p = lo + (uintptr_t)(off + (int64_t)((i0 + i) * stride));
+        const uint32_t d = (uint32_t)(p & 15u);
+        const uint4 *A = reinterpret_cast<const uint4 *>(p - d);
+        whole[i] = p - d >= lo && p - d + 16u * (CH + (d ? 1u : 0u)) <= hi;
+        if (whole[i]) {
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+                set_vec(v[i], q, __ldg(A + q));
+            if (d)
+                set_vec(v[i], CH, __ldg(A + CH));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        uint32_t P[4];
+        const int64_t at = off + (int64_t)((i0 + i) * stride);
+        if (whole[i]) {
+            const uint32_t d = (uint32_t)((lo + (uintptr_t)at) & 15u);
+            uint32_t c[4 * CH];
+            if (d) {
+                join_unit<CH>(v[i], d, c);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4 * CH; ++q)
+                    c[q] = v[i][q];
+            }
+            get_unit<CH>(c, make_sel(CH, 0), P);
+        } else {
+            const uint8_t *p = a.src + at;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t b[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    b[x] = 4u * q + x >= t && 4u * q + x < e ? (uint32_t)__ldg(p + (4 * q + x) * CH) : 0u;
+                P[q] = __byte_perm(__byte_perm(b[0], b[1], 0x0040u),
+                                   __byte_perm(b[2], b[3], 0x0040u), 0x5410u);
+            }
+        }
+        take_pairs(M, P, i0 + i);
+    }
+}
+
+// Pairs of the plane bytes of a unit's words (pair t in byte t%4 of P[t/4]), one
+// shift and one masked merge per pixel: with the byte position at compile time
+// faster here than gathering by byte_perm.
+template <int CH, int PLANE>
+__device__ __forceinline__ void get_pairs(const uint32_t (&w)[4 * CH], uint32_t (&P)[4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        P[q] = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int at = (4 * q + j) * CH + PLANE;
+            P[q] |= ((w[at >> 2] >> (8 * (at & 3))) & 3u) << (8 * j);
+        }
+    }
+}
+
+// Runs k = k_first + i*step < k_end of an aligned layout's full rows, GA
+// quarters' vectors at a time.
+template <int CH, int PLANE, int GA>
+__device__ __forceinline__ void full_runs(const View &a, uint64_t k_first, uint64_t k_end,
+                                          uint32_t step)
+{
+    const uint32_t rpr = a.Q / 16u, W16 = a.W / 16u;
+    const uint32_t stride = rpr * CH; // vectors from quarter to quarter
+    // row and block of the run, kept by additions
+    uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
+    const uint32_t dr = step / rpr, db = step - dr * rpr;
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src);
+    uint4 *out = reinterpret_cast<uint4 *>(a.msg_out);
+    for (uint64_t k = k_first; k < k_end; k += step) {
+        const uint4 *A = src + ((uint64_t)r * W16 + b) * CH;
+        uint32_t M[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int i = 0; i < 4; i += GA) {
+            uint32_t v[GA][4 * CH];
+#pragma unroll
+            for (int x = 0; x < GA; ++x)
 #pragma unroll
                 for (int q = 0; q < CH; ++q)
-                    c[i][q] = __ldcs(u + q);
-            }
-            uint32_t M[4] = {0u, 0u, 0u, 0u};
+                    set_vec(v[x], q, __ldcs(A + (uint64_t)(i + x) * stride + q));
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                uint32_t P[4] = {0u, 0u, 0u, 0u};
+            for (int x = 0; x < GA; ++x) {
+                uint32_t P[4];
                 if constexpr (CH == 1) {
-                    P[0] = c[i][0].x & 0x03030303u;
-                    P[1] = c[i][0].y & 0x03030303u;
-                    P[2] = c[i][0].z & 0x03030303u;
-                    P[3] = c[i][0].w & 0x03030303u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        P[q] = v[x][q] & 0x03030303u;
                 } else {
-                    get_pairs<CH, PLANE>(c[i], P);
+                    get_pairs<CH, PLANE>(v[x], P);
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    M[q] |= P[q] << (2 * i);
+                    M[q] |= P[q] << (2 * (i + x));
             }
-            if (((uintptr_t)mp & 15u) == 0) {
+        }
+        out[k] = make_uint4(M[0], M[1], M[2], M[3]);
+        rc_add(r, b, dr, db, rpr);
+    }
+}
+
+// Extraction over runs k = k_first + i*step < k_end: those of an aligned
+// layout's full rows GA quarters' vectors at a time, then all others G (each
+// part with an index of its own: one carried from the first to the second cost
+// the first its registers, 300 video frames 199 against 180 us).
+template <int CH, int GA, int G>
+__device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, uint64_t k_end,
+                                             uint32_t step)
+{
+    if (k_first >= k_end)
+        return;
+    if (runs_aligned(a)) {
+        const uint64_t full = (uint64_t)(a.L_last == a.Q ? a.R : a.R - 1) * (a.Q / 16u);
+        const uint64_t ke = k_end < full ? k_end : full;
+        switch (CH == 1 ? 0u : a.plane) {
+        case 0: full_runs<CH, 0, GA>(a, k_first, ke, step); break;
+        case 1: full_runs<CH, CH == 1 ? 0 : 1, GA>(a, k_first, ke, step); break;
+        case 2: full_runs<CH, CH == 1 ? 0 : 2, GA>(a, k_first, ke, step); break;
+        default: full_runs<CH, CH == 4 ? 3 : 0, GA>(a, k_first, ke, step); break;
+        }
+        if (k_end <= full)
+            return;
+        if (k_first < full) // the first run past the full rows
+            k_first += (full - k_first + step - 1) / step * step;
+        if (k_first >= k_end)
+            return;
+    }
+    // row and block of the run, kept by additions
+    const uint32_t rpr = run_row(a);
+    uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
+    const uint32_t dr = step / rpr, db = step - dr * rpr;
+    const uint64_t C = (uint64_t)a.W * a.H * CH;
+    for (uint64_t k = k_first; k < k_end; k += step) {
+        const uint32_t L = row_len(a, r);
+        uint8_t *mrow = a.msg_out + (uint64_t)r * a.Q;
+        const int64_t j0 = 16ll * b - (int64_t)((uintptr_t)mrow & 15u); // row byte of the block's first
+        if (j0 < (int64_t)L) {
+            const uint32_t t = j0 < 0 ? (uint32_t)-j0 : 0u;
+            const uint32_t e = (int64_t)L - j0 < 16 ? (uint32_t)(L - j0) : 16u;
+            const int64_t off = ((int64_t)((uint64_t)r * a.W) + j0) * CH + a.plane;
+            uint32_t M[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < 4; i += G)
+                run_quarters<CH, G>(a, C, off, (uint64_t)L * CH, i, t, e, M);
+            uint8_t *mp = mrow + j0;
+            if (e - t == 16u) {
                 *reinterpret_cast<uint4 *>(mp) = make_uint4(M[0], M[1], M[2], M[3]);
             } else {
 #pragma unroll
-                for (int t = 0; t < 16; ++t)
-                    mp[t] = (uint8_t)(M[t >> 2] >> (8 * (t & 3)));
-            }
-        } else {
-            const uint32_t n = L - j0 < 16u ? L - j0 : 16u;
-            for (uint32_t t = 0; t < n; ++t) {
-                uint32_t B = 0;
+                for (int q = 0; q < 4; ++q) {
+                    if (t <= 4u * q && e >= 4u * q + 4u) {
+                        reinterpret_cast<uint32_t *>(mp)[q] = M[q];
+                    } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    B |= (uint32_t)(a.src[(prow + (uint64_t)L * i + j0 + t) * CH + PLANE] & 3u)
-                         << (2 * i);
-                mp[t] = (uint8_t)B;
+                        for (uint32_t x = 4u * q; x < 4u * q + 4u; ++x)
+                            if (x >= t && x < e)
+                                mp[x] = (uint8_t)(M[q] >> (8 * (x & 3u)));
+                    }
+                }
             }
         }
+        rc_add(r, b, dr, db, rpr);
     }
 }
 
@@ -777,23 +986,6 @@ __device__ __forceinline__ void rows_extract(const View &a, uint32_t r_first, ui
                 mrow[j] = (uint8_t)B;
             }
         }
-    }
-}
-
-// Runtime (channels, plane) -> the templated run routine.
-__device__ __forceinline__ void runs_extract_any(const View &a, uint64_t k_first, uint64_t k_end,
-                                                 uint64_t step)
-{
-    switch (a.channels * 4 + a.plane) {
-    case 4: runs_extract<1, 0>(a, k_first, k_end, step); break;
-    case 12: runs_extract<3, 0>(a, k_first, k_end, step); break;
-    case 13: runs_extract<3, 1>(a, k_first, k_end, step); break;
-    case 14: runs_extract<3, 2>(a, k_first, k_end, step); break;
-    case 16: runs_extract<4, 0>(a, k_first, k_end, step); break;
-    case 17: runs_extract<4, 1>(a, k_first, k_end, step); break;
-    case 18: runs_extract<4, 2>(a, k_first, k_end, step); break;
-    case 19: runs_extract<4, 3>(a, k_first, k_end, step); break;
-    default: break;
     }
 }
 

@@ -108,55 +108,6 @@ __device__ __forceinline__ void embed_res(const KView &a, bool stats)
     }
 }
 
-// Changed bytes and squared error of a unit's 16 carrying bytes (c before,
-// o after, d = o ^ c, differences in the low K bits only), summed in 32 bits
-// per unit.  A byte changed when any of its low K bits did (the packing and
-// the per-field test are below).  With K = 1 every change is +-1, so the
-// squared error equals the count.
-template <int K>
-__device__ __forceinline__ void unit_stats(const uint32_t (&o)[4], const uint32_t (&c)[4],
-                                           const uint32_t (&d)[4], uint32_t kmul,
-                                           unsigned long long &changed,
-                                           unsigned long long &sse)
-{
-    constexpr uint32_t BM = ((1u << K) - 1u) * 0x01010101u;
-    uint32_t n, s = 0;
-    static_assert(K >= 1 && K <= 4, "one to four bits per byte");
-    if constexpr (K <= 2) {
-        // the four words' K-bit changes in disjoint bit ranges of each byte
-        // (word i at bits K*i), joined by multiply-adds, then one fold
-        // Horner in kmul = 1 << K: multiply-adds (FMA pipe), not shifts on
-        // the busy ALU pipe; kmul comes from the launch arguments so the
-        // compiler keeps the multiplies
-        const uint32_t acc0 = ((d[3] * kmul + d[2]) * kmul + d[1]) * kmul + d[0];
-        uint32_t acc = acc0;
-        if (K == 2)
-            acc = (acc | (acc >> 1)) & 0x55555555u;
-        n = __popc(acc);
-    } else {
-        // k = 3, 4: two words per byte (word 2j+1 at bit K), then a field is
-        // nonzero when its top bit is set or its low K-1 bits plus all ones
-        // carry into the top bit (no carry leaves a field)
-        constexpr uint32_t LOW = K == 4 ? 0x77777777u : 0x1B1B1B1Bu;
-        constexpr uint32_t TOP = K == 4 ? 0x88888888u : 0x24242424u;
-        const uint32_t a01 = d[1] * kmul + d[0], a23 = d[3] * kmul + d[2];
-        n = __popc((a01 | ((a01 & LOW) + LOW)) & TOP) + __popc((a23 | ((a23 & LOW) + LOW)) & TOP);
-    }
-    if (K > 1) {
-        uint32_t ab = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { // sum of (a - b)^2 = a.a + b.b - 2 a.b over the fields
-            const uint32_t fa = o[i] & BM, fb = c[i] & BM;
-            s = __dp4a(fa, fa, s);
-            s = __dp4a(fb, fb, s);
-            ab = __dp4a(fa, fb, ab);
-        }
-        s -= 2u * ab;
-    }
-    changed += n;
-    sse += K > 1 ? s : n;
-}
-
 // The one vector where the stream ends, field by field (a call of its own
 // keeps the hot loop's registers low).
 __device__ __noinline__ uint4 stream_end_vector(const KView &a, uint64_t v, uint4 c)
