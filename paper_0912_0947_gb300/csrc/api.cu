@@ -530,12 +530,14 @@ int stego_changed_bytes(const uint8_t *d_a, const uint8_t *d_b, uint64_t n, uint
     if (overlap(d_out2, 2 * sizeof(uint64_t), d_a, n) || overlap(d_out2, 2 * sizeof(uint64_t), d_b, n))
         return STEGO_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(d_out2, 0, 2 * sizeof(uint64_t), s) != cudaSuccess)
+    // the totals go through the stream's slot, or into zeroed words
+    StatSlot *slot = n ? stats_slot(s) : nullptr;
+    if (!slot && cudaMemsetAsync(d_out2, 0, 2 * sizeof(uint64_t), s) != cudaSuccess)
         return STEGO_E_CUDA;
     if (n == 0)
         return STEGO_OK;
     const Shape sh = shape_for(STEGO_OP_CHANGED, nullptr);
-    return cuda_status(changed_bytes(d_a, d_b, n, reinterpret_cast<unsigned long long *>(d_out2), sh, s));
+    return cuda_status(changed_bytes(d_a, d_b, n, reinterpret_cast<unsigned long long *>(d_out2), sh, s, slot));
 }
 
 int stego_pointer_kind(const void *p, int *kind, int *device_accessible)

@@ -174,10 +174,11 @@ cudaError_t s1_extract_bulk(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_
                             uint64_t raw_len, bool header, stego_result *res, const Shape &sh,
                             cudaStream_t s);
 
-// Changed-byte count and SSE of two arrays into out2[0..1] (zeroed by the
-// caller).
+// Changed-byte count and SSE of two arrays into out2[0..1] (through the
+// stream's slot; without one they have been zeroed by the caller).
 cudaError_t changed_bytes(const uint8_t *a, const uint8_t *b, uint64_t n,
-                          unsigned long long *out2, const Shape &sh, cudaStream_t s);
+                          unsigned long long *out2, const Shape &sh, cudaStream_t s,
+                          StatSlot *slot);
 
 // One thread writes a whole result (calls that launch no other kernel).
 cudaError_t write_result(stego_result *res, uint64_t msg_bytes, int status, cudaStream_t s);
@@ -264,19 +265,6 @@ __device__ __forceinline__ void block_stats(unsigned long long a, unsigned long 
             atomicExch(&slot->arrived, 0u);
         }
     }
-}
-
-// Changed-byte count and squared error of one 32-bit word pair (four bytes).
-__device__ __forceinline__ void word_stats(uint32_t x, uint32_t y, unsigned long long &changed,
-                                           unsigned long long &sse)
-{
-    uint32_t d = x ^ y;
-    d |= d >> 4; // fold each byte's eight bits into its bit 0
-    d |= d >> 2;
-    d |= d >> 1;
-    changed += __popc(d & 0x01010101u);
-    const uint32_t a = __vabsdiffu4(x, y);
-    sse += __dp4a(a, a, 0u);
 }
 
 // Changed bytes and squared error of a unit's 16 carrying bytes (c before,
