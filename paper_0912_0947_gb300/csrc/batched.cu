@@ -215,8 +215,8 @@ __global__ void prep_embed(const stego_desc *descs, uint32_t n, stego_result *re
             const uint64_t rows_per_tile = rows_for(D, tile_bytes);
             const p2::View v = p2::make_view(nullptr, nullptr, D.geom.width, D.geom.height, ch,
                                              D.geom.plane, nullptr, nullptr, D.msg_bytes);
-            p2::Flat f;
-            const bool flat = p2::make_flat(D.cover, D.stego, D.cover_bytes, ch, D.geom.plane, true, f);
+            Flat f;
+            const bool flat = p2::plan_units(D.cover, D.stego, D.cover_bytes, ch, D.geom.plane, true, f);
             if (flat && (!inplace || (d_aligned16(D.cover) && D.geom.width % 16u == 0))) {
                 // one-pass units, for 1, 3 or 4 channels, any row length and
                 // any addresses; in place (rows of whole vectors, 16-byte
@@ -227,7 +227,7 @@ __global__ void prep_embed(const stego_desc *descs, uint32_t n, stego_result *re
                 inf.mode = inplace ? kP2UnitsInPlace : kP2Units;
                 inf.per_tile = (uint32_t)per;
                 inf.n_bytes = units;
-                inf.nunits = f.nunits;
+                inf.nunits = (uint32_t)f.nunits;
                 inf.flat = f.h | (f.d << 16) | (f.ph << 24);
                 tiles = units ? (units + per - 1) / per : 1u; // (at least the edge bytes)
             } else if (!inplace) {
@@ -569,7 +569,7 @@ __device__ __forceinline__ void claim_loop(const unsigned long long *start,
 // were its loads and stores).
 struct PaperJob {
     p2::View v;
-    p2::Flat f;
+    Flat f;
 };
 
 __device__ __forceinline__ const PaperJob &paper_job(const stego_desc &D, const DescInfo &inf,
@@ -598,7 +598,7 @@ __device__ __forceinline__ const PaperJob &paper_job(const stego_desc &D, const 
         job.f.x0 = inf.channels == 1 ? job.f.h
                                      : (job.f.h + job.f.ph - inf.plane) / inf.channels;
         job.f.nunits = inf.nunits;
-        job.f.sel = p2::make_sel(inf.channels, job.f.ph);
+        job.f.sel = make_sel(inf.channels, job.f.ph);
     }
     __syncthreads();
     return job;

@@ -29,7 +29,7 @@ using p2::View;
 
 struct P2Args {
     View v;
-    p2::Flat f;
+    Flat f;
     stego_result *res;
     StatSlot *slot;
 };
@@ -76,11 +76,11 @@ __global__ void __launch_bounds__(kUnitThreads, CH == 4 ? 2 : CH == 1 ? 5 : 3) p
     if constexpr (CH > 1) {
         __shared__ uint4 stage[p2::stage_vectors<CH>()];
         p2::units_embed_async<CH, STATS, SHIFTED, INPLACE>(
-            a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x, a.f.nunits, gridDim.x * blockDim.x,
+            a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x, (uint32_t)a.f.nunits, gridDim.x * blockDim.x,
             changed, sse, stage);
     } else {
         p2::units_embed<CH, STATS, kUnitsPerThread, INPLACE>(
-            a.v, a.f, blockIdx.x * blockDim.x * kUnitsPerThread + threadIdx.x, a.f.nunits,
+            a.v, a.f, blockIdx.x * blockDim.x * kUnitsPerThread + threadIdx.x, (uint32_t)a.f.nunits,
             gridDim.x * blockDim.x * kUnitsPerThread, changed, sse);
     }
     if (STATS)
@@ -197,7 +197,7 @@ bool p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
                     cudaStream_t s, StatSlot *slot, cudaError_t *err)
 {
     P2Args a = make_args(cover, stego, g, msg, nullptr, N, res);
-    if (!p2::make_flat(cover, stego, (uint64_t)g.width * g.height * g.channels, g.channels,
+    if (!p2::plan_units(cover, stego, (uint64_t)g.width * g.height * g.channels, g.channels,
                        g.plane, false, a.f))
         return false;
     a.slot = stats ? slot : nullptr;
@@ -219,7 +219,7 @@ cudaError_t p2_embed(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
     P2Args a = make_args(cover, stego, g, msg, nullptr, N, res);
     a.slot = stats ? slot : nullptr;
     if (cover == stego && inplace_units_ok(stego, g) &&
-        p2::make_flat(cover, stego, (uint64_t)g.width * g.height * g.channels, g.channels,
+        p2::plan_units(cover, stego, (uint64_t)g.width * g.height * g.channels, g.channels,
                       g.plane, false, a.f)) {
         // in place over the units with carrying pixels (cut inside the
         // kernel): whole vectors instead of one byte access per plane byte

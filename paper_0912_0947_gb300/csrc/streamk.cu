@@ -11,16 +11,19 @@
 // all bytes is handled by stream1.cu.
 //
 // Kernels:
-//   embedk_units<K,CH,PLANE,STATS>  16-byte aligned cover and stego, all
-//       bytes (CH = 1) or one plane of 3 or 4 channels: a unit of 16
-//       carrying bytes (CH vectors of the cover) carries 16K stream bits =
-//       stream bytes [2Ku, 2Ku+2K), assembled big-endian into one 64-bit
-//       word and cut into 16 K-bit fields; out of place the whole cover
-//       moves once, 2C + |S| bytes.
+//   embedk_units<K,STATS,FLAT>, embedk_units_async<K,CH,STATS,FLAT>  all bytes,
+//       or one plane of 1, 3 or 4 channels: a unit of 16 carrying bytes (CH
+//       vectors of the stego) carries 16K stream bits, assembled big-endian
+//       into one 64-bit word and cut into 16 K-bit fields; out of place the
+//       whole cover moves once, 2C + |S| bytes.  FLAT: buffers at any addresses
+//       (units from the stego's 128-byte boundary on, see Flat; the stream cut
+//       at any bit); else both 16-byte aligned, where unit u carries stream
+//       bytes [2Ku, 2Ku + 2K).
 //   embedk_bytes<STATS>  any alignment, any k, either carrying order: one
-//       thread per carrying byte (out of place with one plane, after a copy
-//       of the cover).
-//   extractk_units<K,CH,PLANE>  16-byte aligned stego, same layouts.
+//       thread per carrying byte (other channel counts, one plane in place at
+//       an odd address, covers of less than a few vectors; out of place with
+//       one plane, after a copy of the cover).
+//   extractk_units<K,CH,FLAT>  same layouts; FLAT: a stego at any address.
 //   extractk_bytes  any alignment, any k, either carrying order.
 // The header's 32 bits are read by warp 0 of each CTA: lane l loads stream
 // bit l from its carrying byte and one ballot gathers them.
@@ -28,6 +31,7 @@
 
 #include "async_copy.cuh"
 #include "s1_device.cuh"
+#include "unit_device.cuh"
 
 namespace stego {
 namespace {
@@ -58,6 +62,10 @@ struct KView {
     StatSlot *slot;       // embed: per-stream statistics slot or nullptr
     uint32_t kmul;        // embed: 1 << k (a multiplier the compiler cannot see)
     uint32_t pad;
+    Flat f;               // the units (f.nunits: those embedded; extract: of a FLAT launch
+                          // the whole vectors' units, from u_lo on)
+    uint64_t edge_end;    // embed: end of the cover bytes processed
+    uint64_t u_lo;        // extract, FLAT: first unit whose vectors lie in the stego
 };
 
 __device__ __forceinline__ uint64_t carry_pos(const KView &a, uint64_t x)
@@ -110,12 +118,12 @@ __device__ __forceinline__ void embed_res(const KView &a, bool stats)
 
 // The one vector where the stream ends, field by field (a call of its own
 // keeps the hot loop's registers low).
-__device__ __noinline__ uint4 stream_end_vector(const KView &a, uint64_t v, uint4 c)
+__device__ __noinline__ uint4 stream_end_vector(const KView &a, uint64_t x, uint4 c)
 {
     uint32_t ow[4] = {c.x, c.y, c.z, c.w};
     for (int t = 0; t < 16; ++t) {
         uint32_t fv, fm;
-        field_of(a, v * 16u + t, fv, fm);
+        field_of(a, x + t, fv, fm);
         const uint32_t s = 8 * (t & 3);
         ow[t >> 2] = (ow[t >> 2] & ~(fm << s)) | ((fv & fm) << s);
     }
@@ -162,74 +170,59 @@ __device__ __forceinline__ uint64_t stream_window(const KView &a, uint64_t v)
     return X;
 }
 
+// The 16K stream bits of the carrying bytes x .. x + 15 for any x, in
+// stream_window's form: the aligned message words around the 2K or 2K + 1
+// stream bytes that hold them, byte-shifted, reversed and cut at bit K*x % 8;
+// byte by byte where those words are not all inside the message.
+template <int K>
+__device__ __forceinline__ uint64_t stream_window_at(const KView &a, uint64_t x)
+{
+    constexpr int NW = K >= 3 ? 3 : 2; // words that hold 3 + 2K + 1 bytes
+    const uint64_t b0 = x * K, q = b0 >> 3;
+    const uint32_t s = (uint32_t)(b0 & 7u);
+    const uint64_t hb = a.header ? 4u : 0u;
+    const uintptr_t p = (uintptr_t)a.msg + (uintptr_t)(q - hb);
+    const uint32_t al = (uint32_t)(p & 3u);
+    uint32_t hi, lo, more; // stream bytes q .. q + 3, q + 4 .. q + 7 (first on top), q + 8
+    if (q >= hb + al && q - hb - al + 4u * NW <= a.slen - hb) {
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(p - al);
+        uint32_t v[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            v[i] = i < NW ? __ldg(w + i) : 0u;
+        hi = __byte_perm(__funnelshift_r(v[0], v[1], 8 * al), 0u, 0x0123u);
+        lo = __byte_perm(__funnelshift_r(v[1], v[2], 8 * al), 0u, 0x0123u);
+        more = v[2] >> (8 * al);
+    } else {
+        hi = lo = more = 0u;
+#pragma unroll 1
+        for (int i = 0; i < 9; ++i) { // shifted in from below
+            hi = __funnelshift_l(lo, hi, 8);
+            lo = __funnelshift_l(more << 24, lo, 8);
+            more = i < 2 * K + 1 ? sbyte(a, q + i) : 0u;
+        }
+    }
+    const uint32_t h = __funnelshift_l(lo, hi, s), l = __funnelshift_l(more << 24, lo, s);
+    if constexpr (K == 3)
+        return ((uint64_t)(h >> 8) << 32) | ((h & 0xFFu) << 16) | (l >> 16);
+    else if constexpr (K == 4)
+        return ((uint64_t)h << 32) | l;
+    else
+        return (uint64_t)h << 32;
+}
+
 // A unit is 16 consecutive carrying bytes: 16 consecutive cover bytes (all
 // bytes, CH = 1) or the plane bytes of 16 consecutive pixels (CH = 3 or 4
-// channels, plane PLANE), i.e. CH 16-byte vectors of the cover.  Pixel t's
-// plane byte is unit byte t*CH + PLANE, a compile-time position, so the 16
-// carrying bytes are gathered into one 16-byte value, transformed as one
-// vector of the all-bytes layout, and the change is XORed back.
+// channels), i.e. CH 16-byte vectors.  Its 16 carrying bytes are gathered into
+// one 16-byte value, transformed as one vector of the all-bytes layout, and
+// the change is XORed back.
 template <int CH>
 __device__ __forceinline__ void load_unit(const uint8_t *base, uint64_t u, uint32_t (&w)[4 * CH])
 {
     const uint4 *p = reinterpret_cast<const uint4 *>(base) + u * CH;
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-        const uint4 c = __ldcs(p + j);
-        w[4 * j] = c.x;
-        w[4 * j + 1] = c.y;
-        w[4 * j + 2] = c.z;
-        w[4 * j + 3] = c.w;
-    }
-}
-
-template <int CH>
-__device__ __forceinline__ void store_unit(uint8_t *base, uint64_t u, const uint32_t (&w)[4 * CH])
-{
-    uint4 *p = reinterpret_cast<uint4 *>(base) + u * CH;
-#pragma unroll
     for (int j = 0; j < CH; ++j)
-        __stcs(p + j, make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
-}
-
-// The unit's 16 carrying bytes, byte t of word t/4 = carrying byte t.
-template <int CH, int PLANE>
-__device__ __forceinline__ void gather_unit(const uint32_t (&w)[4 * CH], uint32_t (&g)[4])
-{
-    if constexpr (CH == 1) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            g[i] = w[i];
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            g[i] = 0;
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                const int pos = (4 * i + l) * CH + PLANE; // unit byte of carrying byte 4i+l
-                g[i] |= ((w[pos >> 2] >> (8 * (pos & 3))) & 0xFFu) << (8 * l);
-            }
-        }
-    }
-}
-
-// XOR of carrying-byte differences d (gathered order) into the unit's words.
-template <int CH, int PLANE>
-__device__ __forceinline__ void scatter_xor(uint32_t (&w)[4 * CH], const uint32_t (&d)[4])
-{
-    if constexpr (CH == 1) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            w[i] ^= d[i];
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                const int pos = (4 * i + l) * CH + PLANE;
-                w[pos >> 2] ^= ((d[i] >> (8 * l)) & 0xFFu) << (8 * (pos & 3));
-            }
-        }
-    }
+        set_vec(w, j, __ldcs(p + j));
 }
 
 // Word i (carrying bytes 4i..4i+3, field in each byte's low K bits) of a
@@ -329,98 +322,117 @@ __device__ __forceinline__ void unit_window3(const uint32_t (&g)[4], uint32_t &v
     v23 = (t[2] << 12) | (t[3] & 0xFFFu);
 }
 
-// Units each thread keeps in flight per loop iteration.  A plane unit is
-// already CH vectors; all-bytes units are single vectors, of which the
+// Units each thread of an extract keeps in flight per loop iteration.  A plane
+// unit is already CH vectors; all-bytes units are single vectors, of which the
 // extract batches four (measured on the 201 MB cover, k = 2: 43.0 us
 // against 45.1 us with one, while one is fastest for the embed: 101.4 us
 // against 114.7 us with two and 148.5 us with four).
-constexpr int kEmbedAllBytesUnits = 1;
 constexpr int kExtractAllBytesUnits = 4;
-template <int CH, bool EMBED>
+template <int CH>
 __host__ __device__ constexpr int units_per_iter()
 {
-    return CH == 1 ? (EMBED ? kEmbedAllBytesUnits : kExtractAllBytesUnits) : 1;
+    return CH == 1 ? kExtractAllBytesUnits : 1;
 }
 
-// Embed over units (cover and stego 16-byte aligned): U units per thread
-// per iteration (lane-interleaved), each unit's 16K stream bits = stream
-// bytes [2Ku, 2Ku + 2K) loaded as one big-endian word, all loads issued
-// before any arithmetic.  Units wholly past the stream are copied.
-// Carrying bytes after the last whole unit (fewer than 16) are done by
-// block 0 byte by byte.
-template <int K, int CH, int PLANE, bool STATS>
-__global__ void __launch_bounds__(512, K >= 3 ? 3 : 0) embedk_units(KView a)
+// Bytes outside the units, [0, f.h) and [f.h + 16*CH*nunits, edge_end), by the
+// calling CTA: plane bytes take their field, the other bytes of those pixels
+// are copied (in place only what changes is written).
+template <int CH, bool STATS>
+__device__ __forceinline__ void embedk_edges(const KView &a, unsigned long long &changed,
+                                             unsigned long long &sse)
 {
-    grid_dependency_wait(); // launched dependent: nothing is touched before
-    allow_dependents();
-    constexpr int U = units_per_iter<CH, true>();
-    constexpr uint32_t MASK = (1u << K) - 1u;
-    constexpr uint32_t BYTEMASK = MASK * 0x01010101u;
-    unsigned long long changed = 0, sse = 0;
-    embed_res(a, STATS);
-    const uint64_t nunits = a.n_carry >> 4;
-    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x * U + threadIdx.x; u0 < nunits;
-         u0 += (uint64_t)gridDim.x * blockDim.x * U) {
-        uint32_t w[U][4 * CH];
-        uint64_t X[U];
-#pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u < nunits)
-                load_unit<CH>(a.cover, u, w[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            X[r] = (u < nunits && u < a.full_units) ? stream_window<K>(a, u) : 0ull;
-        }
-#pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u >= nunits)
-                continue;
-            if (u < a.part_units) {
-                uint32_t c[4], o[4];
-                gather_unit<CH, PLANE>(w[r], c);
-                if (u < a.full_units) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        o[i] = (c[i] & ~BYTEMASK) | unit_fields<K>(X[r], i);
-                } else {
-                    const uint4 e = stream_end_vector(a, u, make_uint4(c[0], c[1], c[2], c[3]));
-                    o[0] = e.x;
-                    o[1] = e.y;
-                    o[2] = e.z;
-                    o[3] = e.w;
-                }
-                uint32_t d[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    d[i] = o[i] ^ c[i];
-                if (STATS)
-                    unit_stats<K>(o, c, d, a.kmul, changed, sse);
-                scatter_xor<CH, PLANE>(w[r], d);
-            }
-            store_unit<CH>(a.stego, u, w[r]);
-        }
-    }
-    // cover bytes of the carrying bytes after the last whole unit: plane
-    // bytes take their field, the other bytes of those pixels are copied
-    if (blockIdx.x == 0 && threadIdx.x < (uint32_t)(a.n_carry & 15u) * CH) {
-        const uint64_t pbyte = ((a.n_carry >> 4) << 4) * CH + threadIdx.x;
-        const uint32_t cb = a.cover[pbyte];
+    const uint64_t t0 = a.f.h + 16u * CH * a.f.nunits;
+    const uint32_t nt = a.edge_end > t0 ? (uint32_t)(a.edge_end - t0) : 0u;
+    for (uint32_t e = threadIdx.x; e < a.f.h + nt; e += blockDim.x) {
+        const uint64_t k = e < a.f.h ? e : t0 + (e - a.f.h);
+        const uint32_t cb = a.cover[k];
         uint32_t ob = cb;
-        if (threadIdx.x % CH == PLANE) {
+        if (k % CH == a.plane) {
             uint32_t fv, fm;
-            field_of(a, pbyte / CH, fv, fm);
+            field_of(a, k / CH, fv, fm);
             ob = (cb & ~fm) | (fv & fm);
         }
-        a.stego[pbyte] = (uint8_t)ob;
+        if (ob != cb || a.stego != a.cover)
+            a.stego[k] = (uint8_t)ob;
         if (STATS) {
             const uint32_t dd = ob > cb ? ob - cb : cb - ob;
             changed += dd != 0;
             sse += dd * dd;
         }
+    }
+}
+
+// The 16 carrying bytes c of unit u (first carrying byte x) -> o, its stream
+// window X read when the unit lies wholly inside the stream.
+template <int K>
+__device__ __forceinline__ void embed_fields(const KView &a, uint64_t u, uint64_t x, uint64_t X,
+                                             const uint32_t (&c)[4], uint32_t (&o)[4])
+{
+    constexpr uint32_t BYTEMASK = ((1u << K) - 1u) * 0x01010101u;
+    if (u < a.full_units) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            o[i] = (c[i] & ~BYTEMASK) | unit_fields<K>(X, i);
+    } else {
+        const uint4 e = stream_end_vector(a, x, make_uint4(c[0], c[1], c[2], c[3]));
+        o[0] = e.x;
+        o[1] = e.y;
+        o[2] = e.z;
+        o[3] = e.w;
+    }
+}
+
+// Embed over all-bytes units, single vectors, one per thread and iteration
+// (see kExtractAllBytesUnits).  Units wholly past the stream are copied.  FLAT:
+// a cover at another address mod 16 than the stego is read as the two vectors
+// around the unit's bytes (the second is the neighbour's first: an L1 hit).
+// All bytes at k = 2, 3, 4 are bound by instructions as much as by HBM (ALU pipe
+// 60% at k = 2; 8192x8192x3 77.1 / 84.6 / 83.4 us).  Buffers at odd addresses
+// ran one thread per carrying byte before: 5471x3647x3, cover 13 bytes past a
+// boundary, k = 2, 3, 4: 220 / 215 / 217 -> 31.3 / 34.3 / 34.5 us, both 13 bytes
+// past, k = 2: 220 -> 27.5.  An odd message with aligned covers (byte loads
+// before) 28.8 -> 26.8.
+template <int K, bool STATS, bool FLAT>
+__global__ void __launch_bounds__(512, K >= 3 ? 3 : 0) embedk_units(KView a)
+{
+    grid_dependency_wait(); // launched dependent: nothing is touched before
+    allow_dependents();
+    unsigned long long changed = 0, sse = 0;
+    embed_res(a, STATS);
+    if (blockIdx.x == gridDim.x - 1) // the CTA with the fewest units
+        embedk_edges<1, STATS>(a, changed, sse);
+    const uint64_t nunits = a.f.nunits;
+    const uint4 *__restrict__ src =
+        reinterpret_cast<const uint4 *>(a.cover + (FLAT ? a.f.h - a.f.d : 0u));
+    uint4 *dst = reinterpret_cast<uint4 *>(a.stego + (FLAT ? a.f.h : 0u));
+    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunits;
+         u += (uint64_t)gridDim.x * blockDim.x) {
+        uint32_t w[4];
+        if (FLAT && a.f.d) {
+            uint32_t v[8];
+            set_vec(v, 0, __ldcs(src + u));
+            set_vec(v, 1, __ldcs(src + u + 1));
+            join_unit<1>(v, a.f.d, w);
+        } else {
+            set_vec(w, 0, __ldcs(src + u));
+        }
+        if (u < a.part_units) {
+            const uint64_t x = (FLAT ? a.f.x0 : 0u) + 16u * u;
+            uint64_t X = 0;
+            if (u < a.full_units)
+                X = FLAT ? stream_window_at<K>(a, x) : stream_window<K>(a, u);
+            uint32_t o[4], d[4];
+            embed_fields<K>(a, u, x, X, w, o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                d[i] = o[i] ^ w[i];
+            if (STATS)
+                unit_stats<K>(o, w, d, a.kmul, changed, sse);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                w[i] = o[i];
+        }
+        __stcs(dst + u, get_vec(w, 0));
     }
     if (STATS)
         block_stats(changed, sse, a.res, a.slot);
@@ -432,38 +444,51 @@ __global__ void __launch_bounds__(512, K >= 3 ? 3 : 0) embedk_units(KView a)
 // order, coalesced: a lane's own unit is 16*CH bytes from its neighbour's)
 // and the next units' stream windows on their way to registers.  Each lane
 // then takes its unit from shared memory, embeds it as embedk_units does and
-// writes it back; the warp stores its vectors in memory order.  CTAs of at
-// most kAsyncThreads threads (the staging area holds that many warps).
+// writes it back; the warp stores its vectors in memory order.  FLAT with
+// cover and stego at different addresses mod 16: the stage holds the 32*CH + 1
+// aligned cover vectors around the warp's bytes, of which each lane reads CH +
+// 1.  CTAs of at most kAsyncThreads threads (the staging area holds that many
+// warps).  HBM-bound: k = 2, plane 0 of 8192x8192x3 67.5 us; with the plane's
+// position at run time (one kernel for all) as fast as at compile time (68.9).
+// 3839x2159x3 in packed stacks, k = 3, plane 1 (a copy and a kernel of one
+// thread per carrying byte before): 39.2 -> 14.4 us.
 constexpr int kAsyncThreads = 256;
-template <int K, int CH, int PLANE, bool STATS>
+template <int K, int CH, bool STATS, bool FLAT>
 __global__ void __launch_bounds__(kAsyncThreads) embedk_units_async(KView a)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
     static_assert(CH > 1, "plane units only");
-    constexpr uint32_t MASK = (1u << K) - 1u;
-    constexpr uint32_t BYTEMASK = MASK * 0x01010101u;
-    constexpr uint32_t SV = unit_stage_slots<CH>();
+    constexpr uint32_t SV = unit_stage_slots<CH>() + (FLAT ? 1u : 0u);
     __shared__ uint4 stage[(kAsyncThreads / 32) * 2 * SV];
     uint4 *const sw = stage + (threadIdx.x >> 5) * 2 * SV;
     const uint32_t lane = threadIdx.x & 31u;
     unsigned long long changed = 0, sse = 0;
     embed_res(a, STATS);
-    const uint64_t nunits = a.n_carry >> 4;
-    const uint64_t vend = nunits * CH;
-    const uint4 *__restrict__ cv = reinterpret_cast<const uint4 *>(a.cover);
-    uint4 *const ov = reinterpret_cast<uint4 *>(a.stego);
+    if (blockIdx.x == gridDim.x - 1) // the CTA with the fewest units
+        embedk_edges<CH, STATS>(a, changed, sse);
+    const uint64_t nunits = a.f.nunits;
+    const bool joined = FLAT && a.f.d;
+    const uint64_t vend = nunits * CH;              // vectors written
+    const uint64_t vread = vend + (joined ? 1u : 0u); // and read
+    const uint4 *__restrict__ cv =
+        reinterpret_cast<const uint4 *>(a.cover + (FLAT ? a.f.h - a.f.d : 0u));
+    uint4 *const ov = reinterpret_cast<uint4 *>(a.stego + (FLAT ? a.f.h : 0u));
     const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
     auto issue = [&](uint64_t ub, uint32_t s) { // the warp's vectors from unit ub -> stage s
         const uint64_t v0 = ub * CH;
 #pragma unroll
         for (int j = 0; j < CH; ++j)
-            if (v0 + 32u * j + lane < vend)
+            if (v0 + 32u * j + lane < vread)
                 cp_async16(sw + s * SV + unit_stage_slot<CH>(32u * j + lane), cv + v0 + 32u * j + lane);
+        if (FLAT && lane == 0 && v0 + 32u * CH < vread)
+            cp_async16(sw + s * SV + unit_stage_slot<CH>(32u * CH), cv + v0 + 32u * CH);
         cp_async_commit();
     };
     auto window = [&](uint64_t u) {
-        return (u < nunits && u < a.full_units) ? stream_window<K>(a, u) : 0ull;
+        if (u >= nunits || u >= a.full_units)
+            return (uint64_t)0;
+        return FLAT ? stream_window_at<K>(a, a.f.x0 + 16u * u) : stream_window<K>(a, u);
     };
     uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; // u - lane: the same for the warp
     if (u - lane < nunits) {
@@ -483,40 +508,35 @@ __global__ void __launch_bounds__(kAsyncThreads) embedk_units_async(KView a)
             }
             __syncwarp(); // every lane's copies visible to the warp
             uint4 *const st = sw + s * SV;
-            if (u < nunits && u < a.part_units) {
+            const bool embeds = u < nunits && u < a.part_units;
+            if (joined || embeds) {
                 uint32_t w[4 * CH];
+                if (joined) {
+                    uint32_t v[4 * CH + 4];
 #pragma unroll
-                for (int q = 0; q < CH; ++q) {
-                    const uint4 t = st[unit_stage_slot<CH>(CH * lane + q)];
-                    w[4 * q] = t.x;
-                    w[4 * q + 1] = t.y;
-                    w[4 * q + 2] = t.z;
-                    w[4 * q + 3] = t.w;
+                    for (int q = 0; q <= CH; ++q)
+                        set_vec(v, q, st[unit_stage_slot<CH>(CH * lane + q)]);
+                    join_unit<CH>(v, a.f.d, w);
+                    __syncwarp(); // the neighbour has read this lane's first vector
+                } else {
+#pragma unroll
+                    for (int q = 0; q < CH; ++q)
+                        set_vec(w, q, st[unit_stage_slot<CH>(CH * lane + q)]);
                 }
-                uint32_t c[4], o[4];
-                gather_unit<CH, PLANE>(w, c);
-                if (u < a.full_units) {
+                if (embeds) {
+                    uint32_t c[4], o[4], d[4];
+                    get_unit<CH>(w, a.f.sel, c);
+                    embed_fields<K>(a, u, (FLAT ? a.f.x0 : 0u) + 16u * u, X, c, o);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        o[i] = (c[i] & ~BYTEMASK) | unit_fields<K>(X, i);
-                } else {
-                    const uint4 e = stream_end_vector(a, u, make_uint4(c[0], c[1], c[2], c[3]));
-                    o[0] = e.x;
-                    o[1] = e.y;
-                    o[2] = e.z;
-                    o[3] = e.w;
+                        d[i] = o[i] ^ c[i];
+                    if (STATS)
+                        unit_stats<K>(o, c, d, a.kmul, changed, sse);
+                    xor_unit<CH>(w, a.f.sel, d);
                 }
-                uint32_t d[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    d[i] = o[i] ^ c[i];
-                if (STATS)
-                    unit_stats<K>(o, c, d, a.kmul, changed, sse);
-                scatter_xor<CH, PLANE>(w, d);
 #pragma unroll
                 for (int q = 0; q < CH; ++q)
-                    st[unit_stage_slot<CH>(CH * lane + q)] =
-                        make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                    st[unit_stage_slot<CH>(CH * lane + q)] = get_vec(w, q);
             }
             __syncwarp(); // the rewritten units visible to the storing lanes
             const uint64_t v0 = (u - lane) * CH;
@@ -526,29 +546,11 @@ __global__ void __launch_bounds__(kAsyncThreads) embedk_units_async(KView a)
                     __stcs(ov + v0 + 32u * j + lane, st[unit_stage_slot<CH>(32u * j + lane)]);
             if (!next)
                 break;
-            // stage s is refilled two iterations on, after this lane's reads
-            // of its own memory-order slots above
+            // stage s is refilled two iterations on, after every lane passed
+            // the barriers above and read its own memory-order slots
             X = Xn;
             u = un;
             s ^= 1u;
-        }
-    }
-    // cover bytes of the carrying bytes after the last whole unit: plane
-    // bytes take their field, the other bytes of those pixels are copied
-    if (blockIdx.x == 0 && threadIdx.x < (uint32_t)(a.n_carry & 15u) * CH) {
-        const uint64_t pbyte = ((a.n_carry >> 4) << 4) * CH + threadIdx.x;
-        const uint32_t cb = a.cover[pbyte];
-        uint32_t ob = cb;
-        if (threadIdx.x % CH == PLANE) {
-            uint32_t fv, fm;
-            field_of(a, pbyte / CH, fv, fm);
-            ob = (cb & ~fm) | (fv & fm);
-        }
-        a.stego[pbyte] = (uint8_t)ob;
-        if (STATS) {
-            const uint32_t dd = ob > cb ? ob - cb : cb - ob;
-            changed += dd != 0;
-            sse += dd * dd;
         }
     }
     if (STATS)
@@ -630,6 +632,22 @@ __device__ __forceinline__ int extractk_prologue(const KView &a, uint64_t &len)
     return status;
 }
 
+// Unit u's words: its vectors, or (FLAT) its bytes from the vectors around them.
+template <int CH, bool FLAT>
+__device__ __forceinline__ void read_unit(const KView &a, uint64_t u, uint32_t (&w)[4 * CH])
+{
+    if constexpr (FLAT) {
+        const uint4 *p = reinterpret_cast<const uint4 *>(a.cover - a.f.d) + u * CH;
+        uint32_t v[4 * CH + 4];
+#pragma unroll
+        for (int j = 0; j <= CH; ++j)
+            set_vec(v, j, __ldg(p + j));
+        join_unit<CH>(v, a.f.d, w);
+    } else {
+        load_unit<CH>(a.cover, u, w);
+    }
+}
+
 // k = 3 units of the extract: unit u yields the 6 stream bytes [6u, 6u + 6),
 // so a lane pair (units 2j, 2j + 1) holds 12 consecutive message bytes and
 // writes them as three aligned words: the even lane its first four bytes
@@ -637,11 +655,11 @@ __device__ __forceinline__ int extractk_prologue(const KView &a, uint64_t &len)
 // odd lane its last four.  The loop runs while the warp's first unit is in
 // range, so every lane reaches the shuffle; pairs at the header, at the
 // message's end or on an unaligned output store 16-bit halves or bytes.
-template <int CH, int PLANE>
-__device__ __forceinline__ void extract3_units(const KView &a, uint64_t nunits, uint64_t hb,
-                                               uint64_t sbytes)
+template <int CH, bool FLAT>
+__device__ __forceinline__ void extract3_units(const KView &a, uint64_t ulo, uint64_t nunits,
+                                               uint64_t hb, uint64_t sbytes)
 {
-    constexpr int U = units_per_iter<CH, false>();
+    constexpr int U = units_per_iter<CH>();
     const uint32_t lane = threadIdx.x & 31u;
     const bool odd = (lane & 1u) != 0;
     // stream byte 12j lands at out + 12j - hb: word-aligned for every j or none
@@ -652,8 +670,8 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t nunits, 
 #pragma unroll
         for (int r = 0; r < U; ++r) {
             const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u < nunits) {
-                load_unit<CH>(a.cover, u, w[r]);
+            if (u < nunits && u >= ulo) {
+                read_unit<CH, FLAT>(a, u, w[r]);
             } else {
 #pragma unroll
                 for (int j = 0; j < 4 * CH; ++j)
@@ -664,13 +682,13 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t nunits, 
         for (int r = 0; r < U; ++r) {
             const uint64_t u = u0 + (uint64_t)r * blockDim.x;
             uint32_t g[4], v01, v23;
-            gather_unit<CH, PLANE>(w[r], g);
+            get_unit<CH>(w[r], a.f.sel, g);
             unit_window3(g, v01, v23);
             const uint32_t P = __byte_perm(v01, v23, 0x6012u); // stream bytes 0-3, memory order
             const uint32_t Q = __byte_perm(v23, 0u, 0x4401u);  // stream bytes 4-5
             const uint32_t Pn = __shfl_down_sync(0xFFFFFFFFu, P, 1);
             const uint64_t q2 = 6u * (u & ~1ull); // first stream byte of the pair
-            if (words && (u | 1u) < nunits && q2 >= hb && q2 + 12 <= sbytes) {
+            if (words && (u | 1u) < nunits && (u & ~1ull) >= ulo && q2 >= hb && q2 + 12 <= sbytes) {
                 uint32_t *op = reinterpret_cast<uint32_t *>(a.out + (q2 - hb));
                 if (odd) {
                     op[2] = __byte_perm(P, Q, 0x5432u);
@@ -678,7 +696,7 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t nunits, 
                     op[0] = P;
                     op[1] = __byte_perm(Q, Pn, 0x5410u);
                 }
-            } else if (u < nunits) {
+            } else if (u < nunits && u >= ulo) {
                 const uint64_t q0 = 6u * u; // first stream byte of the unit
                 if (q0 >= hb && q0 + 6 <= sbytes && ((q0 - hb + (uintptr_t)a.out) & 1u) == 0) {
                     unsigned short *op = reinterpret_cast<unsigned short *>(a.out + (q0 - hb));
@@ -698,10 +716,13 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t nunits, 
     }
 }
 
-// Extract over units (stego 16-byte aligned): unit u yields stream bytes
-// [2Ku, 2Ku + 2K); U units per thread per iteration, loads first.  Stream
-// bytes past the last whole unit go bit by bit.
-template <int K, int CH, int PLANE>
+// Extract over units: unit u yields stream bytes [2Ku, 2Ku + 2K); U units per
+// thread per iteration, loads first.  FLAT: a stego at any address, its units
+// read as the CH + 1 aligned vectors around them (3839x2159x3, k = 3, plane 1:
+// 16.6 us bit by bit -> 5.5; 5471x3647x3, all bytes, k = 2, 3: 71 / 104 -> 17.3 /
+// 20.5).  Stream bytes before the
+// first and past the last unit whose vectors lie in the stego go bit by bit.
+template <int K, int CH, bool FLAT>
 __global__ void __launch_bounds__(512) extractk_units(KView a)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
@@ -712,9 +733,14 @@ __global__ void __launch_bounds__(512) extractk_units(KView a)
     const uint64_t hb = a.header ? 4u : 0u;       // stream bytes before the message
     const uint64_t sbytes = len + hb;              // stream bytes to recover
     const uint64_t want = (sbytes + 2 * K - 1) / (2 * K);
-    const uint64_t nunits = want < (a.n_carry >> 4) ? want : (a.n_carry >> 4);
-    for (uint64_t q = 2u * K * nunits + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-         q < sbytes; q += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t nunits = want < a.f.nunits ? want : a.f.nunits;
+    const uint64_t ulo = FLAT ? (a.u_lo < nunits ? a.u_lo : nunits) : 0u;
+    // stream bytes [u0, u1) are the units'; the others one by one
+    const uint64_t u1 = 2u * K * nunits < sbytes ? 2u * K * nunits : sbytes;
+    const uint64_t u0 = 2u * K * ulo < u1 ? 2u * K * ulo : u1;
+    for (uint64_t qq = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; qq < sbytes - (u1 - u0);
+         qq += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t q = qq < u0 ? qq : qq + (u1 - u0);
         if (q < hb)
             continue;
         uint32_t v = 0;
@@ -724,26 +750,26 @@ __global__ void __launch_bounds__(512) extractk_units(KView a)
         a.out[q - hb] = (uint8_t)v;
     }
     if constexpr (K == 3) {
-        extract3_units<CH, PLANE>(a, nunits, hb, sbytes);
+        extract3_units<CH, FLAT>(a, ulo, nunits, hb, sbytes);
         return;
     }
-    constexpr int U = units_per_iter<CH, false>();
-    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x * U + threadIdx.x; u0 < nunits;
-         u0 += (uint64_t)gridDim.x * blockDim.x * U) {
+    constexpr int U = units_per_iter<CH>();
+    for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x * U + threadIdx.x; v0 < nunits;
+         v0 += (uint64_t)gridDim.x * blockDim.x * U) {
         uint32_t w[U][4 * CH];
 #pragma unroll
         for (int r = 0; r < U; ++r) {
-            const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u < nunits)
-                load_unit<CH>(a.cover, u, w[r]);
+            const uint64_t u = v0 + (uint64_t)r * blockDim.x;
+            if (u < nunits && u >= ulo)
+                read_unit<CH, FLAT>(a, u, w[r]);
         }
 #pragma unroll
         for (int r = 0; r < U; ++r) {
-            const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u >= nunits)
+            const uint64_t u = v0 + (uint64_t)r * blockDim.x;
+            if (u >= nunits || u < ulo)
                 continue;
             uint32_t g[4];
-            gather_unit<CH, PLANE>(w[r], g);
+            get_unit<CH>(w[r], a.f.sel, g);
             const uint64_t X = unit_window<K>(g);
             const uint64_t q0 = 2u * K * u; // first stream byte of the unit
             uint8_t *op = a.out + (q0 - hb);
@@ -804,64 +830,45 @@ bool unit_layout(bool plane_only, const stego_geom *g)
     return !plane_only || g->channels == 1 || g->channels == 3 || g->channels == 4;
 }
 
-template <int K, bool STATS>
-const void *embed_units_for(uint32_t ch, uint32_t plane)
+template <int K, bool STATS, bool FLAT>
+const void *embed_units_for(uint32_t ch)
 {
-    if (ch == 1)
-        return (const void *)embedk_units<K, 1, 0, STATS>;
-    if (ch == 3) {
-        switch (plane) {
-        case 0: return (const void *)embedk_units_async<K, 3, 0, STATS>;
-        case 1: return (const void *)embedk_units_async<K, 3, 1, STATS>;
-        default: return (const void *)embedk_units_async<K, 3, 2, STATS>;
-        }
-    }
-    switch (plane) {
-    case 0: return (const void *)embedk_units_async<K, 4, 0, STATS>;
-    case 1: return (const void *)embedk_units_async<K, 4, 1, STATS>;
-    case 2: return (const void *)embedk_units_async<K, 4, 2, STATS>;
-    default: return (const void *)embedk_units_async<K, 4, 3, STATS>;
+    switch (ch) {
+    case 1: return (const void *)embedk_units<K, STATS, FLAT>;
+    case 3: return (const void *)embedk_units_async<K, 3, STATS, FLAT>;
+    default: return (const void *)embedk_units_async<K, 4, STATS, FLAT>;
     }
 }
 
-template <bool STATS>
-const void *embed_units_kernel(uint32_t k, uint32_t ch, uint32_t plane)
+template <bool STATS, bool FLAT>
+const void *embed_units_kernel(uint32_t k, uint32_t ch)
 {
     switch (k) {
-    case 1: return embed_units_for<1, STATS>(ch, plane);
-    case 2: return embed_units_for<2, STATS>(ch, plane);
-    case 3: return embed_units_for<3, STATS>(ch, plane);
-    default: return embed_units_for<4, STATS>(ch, plane);
+    case 1: return embed_units_for<1, STATS, FLAT>(ch);
+    case 2: return embed_units_for<2, STATS, FLAT>(ch);
+    case 3: return embed_units_for<3, STATS, FLAT>(ch);
+    default: return embed_units_for<4, STATS, FLAT>(ch);
     }
 }
 
-template <int K>
-const void *extract_units_for(uint32_t ch, uint32_t plane)
+template <int K, bool FLAT>
+const void *extract_units_for(uint32_t ch)
 {
-    if (ch == 1)
-        return (const void *)extractk_units<K, 1, 0>;
-    if (ch == 3) {
-        switch (plane) {
-        case 0: return (const void *)extractk_units<K, 3, 0>;
-        case 1: return (const void *)extractk_units<K, 3, 1>;
-        default: return (const void *)extractk_units<K, 3, 2>;
-        }
-    }
-    switch (plane) {
-    case 0: return (const void *)extractk_units<K, 4, 0>;
-    case 1: return (const void *)extractk_units<K, 4, 1>;
-    case 2: return (const void *)extractk_units<K, 4, 2>;
-    default: return (const void *)extractk_units<K, 4, 3>;
+    switch (ch) {
+    case 1: return (const void *)extractk_units<K, 1, FLAT>;
+    case 3: return (const void *)extractk_units<K, 3, FLAT>;
+    default: return (const void *)extractk_units<K, 4, FLAT>;
     }
 }
 
-const void *extract_units_kernel(uint32_t k, uint32_t ch, uint32_t plane)
+template <bool FLAT>
+const void *extract_units_kernel(uint32_t k, uint32_t ch)
 {
     switch (k) {
-    case 1: return extract_units_for<1>(ch, plane);
-    case 2: return extract_units_for<2>(ch, plane);
-    case 3: return extract_units_for<3>(ch, plane);
-    default: return extract_units_for<4>(ch, plane);
+    case 1: return extract_units_for<1, FLAT>(ch);
+    case 2: return extract_units_for<2, FLAT>(ch);
+    case 3: return extract_units_for<3, FLAT>(ch);
+    default: return extract_units_for<4, FLAT>(ch);
     }
 }
 
@@ -889,8 +896,6 @@ cudaError_t sk_embed(const uint8_t *cover, uint8_t *stego, uint64_t C, uint32_t 
     a.res = res;
     a.res_msg_bytes = m;
     a.slot = stats ? slot : nullptr;
-    a.full_units = a.t_bits / (16u * k);
-    a.part_units = (a.t_bits + 16u * k - 1) / (16u * k);
     a.msg_w4 = (((uintptr_t)msg - (header ? 4u : 0u)) & 3u) == 0;
     a.msg_w2 = (((uintptr_t)msg - (header ? 4u : 0u)) & 1u) == 0;
     a.kmul = 1u << k;
@@ -898,17 +903,39 @@ cudaError_t sk_embed(const uint8_t *cover, uint8_t *stego, uint64_t C, uint32_t 
     const uint64_t t_carry = (a.t_bits + k - 1) / k; // carrying bytes the stream uses
     const int T = sh.threads;
     void *args[] = {&a};
-    if (aligned16(cover) && aligned16(stego) && unit_layout(plane_only, g)) {
-        // carrying bytes processed: all of them out of place (the rest of
-        // the cover is copied with them), those the stream uses in place
-        a.n_carry = inplace ? t_carry : (plane_only ? (uint64_t)g->width * g->height : C);
-        const void *kern = stats ? embed_units_kernel<true>(k, a.channels, a.plane)
-                                 : embed_units_kernel<false>(k, a.channels, a.plane);
-        const uint64_t nunits = a.n_carry >> 4;
-        const int per_thread = a.channels == 1 ? kEmbedAllBytesUnits : 1;
+    // one plane in place at an odd address keeps to its plane bytes; all else
+    // of these layouts runs in units, in place those the stream fills whole
+    const bool aligned = aligned16(cover) && aligned16(stego);
+    // (the aligned kernel's message loads: words or, at k = 3, halves)
+    const bool msg_ok = k == 1 || (k == 3 ? a.msg_w2 : a.msg_w4);
+    const bool flat = !aligned || !msg_ok;
+    if (unit_layout(plane_only, g) && (aligned || !inplace || a.channels == 1) &&
+        (!flat || make_flat(cover, stego, C, a.channels, a.plane, false, a.f))) {
+        const uint64_t all = plane_only ? (uint64_t)g->width * g->height : C; // carrying bytes
+        a.n_carry = inplace ? t_carry : all;
+        a.edge_end = inplace ? t_carry * a.channels : C;
+        if (!flat) {
+            a.f.h = a.f.d = a.f.x0 = 0;
+            a.f.ph = a.plane;
+            a.f.sel = make_sel(a.channels, a.plane);
+            a.f.nunits = a.n_carry >> 4;
+        } else if (inplace) {
+            const uint64_t whole = t_carry > a.f.x0 ? (t_carry - a.f.x0) >> 4 : 0u;
+            if (whole < a.f.nunits)
+                a.f.nunits = whole;
+            if (a.f.h > a.edge_end)
+                a.f.h = (uint32_t)a.edge_end; // (a stream that ends in the head)
+        }
+        const uint64_t bits0 = (uint64_t)k * a.f.x0; // stream bits before unit 0
+        a.full_units = a.t_bits > bits0 ? (a.t_bits - bits0) / (16u * k) : 0u;
+        a.part_units = a.t_bits > bits0 ? (a.t_bits - bits0 + 16u * k - 1) / (16u * k) : 0u;
+        const void *kern = flat ? (stats ? embed_units_kernel<true, true>(k, a.channels)
+                                         : embed_units_kernel<false, true>(k, a.channels))
+                                : (stats ? embed_units_kernel<true, false>(k, a.channels)
+                                         : embed_units_kernel<false, false>(k, a.channels));
         const int TU = a.channels == 1 ? T : kAsyncThreads; // plane units: the pipeline's CTAs
-        const int grid = persistent_grid(kern, TU, 0, kAnyCtas, nunits ? nunits : 1,
-                                         (uint64_t)TU * per_thread);
+        const int grid = persistent_grid(kern, TU, 0, kAnyCtas, a.f.nunits ? a.f.nunits : 1,
+                                         (uint64_t)TU);
         return launch_dependent(kern, dim3(grid), dim3(TU), args, 0, s);
     }
     if (plane_only && !inplace) {
@@ -951,11 +978,22 @@ cudaError_t sk_extract(const uint8_t *st, uint64_t C, uint32_t k, bool plane_onl
     }
     const int T = sh.threads;
     void *args[] = {&a};
-    if (aligned16(st) && unit_layout(plane_only, g)) {
-        const void *kern = extract_units_kernel(k, a.channels, a.plane);
-        const uint64_t nunits = (max_len + 4 + 2 * k - 1) / (2 * k);
-        const int per_thread = a.channels == 1 ? kExtractAllBytesUnits : 1;
-        const int grid = persistent_grid(kern, T, 0, kAnyCtas, nunits ? nunits : 1,
+    if (unit_layout(plane_only, g)) {
+        const bool flat = !aligned16(st);
+        const uint32_t ch = a.channels;
+        const uint64_t units = (max_len + 4 + 2 * k - 1) / (2 * k);
+        a.f.d = (uint32_t)((uintptr_t)st & 15u);
+        a.f.sel = make_sel(ch, a.plane);
+        a.f.nunits = a.n_carry >> 4;
+        a.u_lo = 0;
+        if (flat) {
+            // units whose CH + 1 vectors lie inside the stego
+            a.u_lo = 1;
+            a.f.nunits = C > 16u - a.f.d ? (C - (16u - a.f.d)) / (16u * ch) : 0u;
+        }
+        const void *kern = flat ? extract_units_kernel<true>(k, ch) : extract_units_kernel<false>(k, ch);
+        const int per_thread = ch == 1 ? kExtractAllBytesUnits : 1;
+        const int grid = persistent_grid(kern, T, 0, kAnyCtas, units ? units : 1,
                                          (uint64_t)T * per_thread);
         return launch_dependent(kern, dim3(grid), dim3(T), args, 0, s);
     }
