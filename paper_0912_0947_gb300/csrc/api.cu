@@ -182,7 +182,7 @@ int sm_count()
 }
 
 cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, void **args,
-                             size_t smem, cudaStream_t s)
+                             size_t smem, cudaStream_t s, uint32_t cluster)
 {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -190,12 +190,19 @@ cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, void **a
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     std::memset(at, 0, sizeof(at));
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    if (cluster > 1) {
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = cluster;
+        at[1].val.clusterDim.y = 1;
+        at[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 

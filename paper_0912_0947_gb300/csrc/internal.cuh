@@ -58,8 +58,9 @@ int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_s
 // before it in the stream is still finishing (its CTAs then wait on the SMs
 // instead of behind the launch).  Only for kernels that call
 // grid_dependency_wait() before their first global memory access.
+// cluster > 1: CTAs per thread block cluster (the grid a multiple of it).
 cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, void **args,
-                             size_t smem, cudaStream_t s);
+                             size_t smem, cudaStream_t s, uint32_t cluster = 1);
 
 // Returns once the grid before this one in the stream has completed and its
 // memory operations are visible (at once when there is none, or when the
