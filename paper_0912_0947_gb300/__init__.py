@@ -218,11 +218,16 @@ def _check(st: int, where: str) -> int:
 
 # -- marshalling helpers -------------------------------------------------------
 
-def _dev_ptr(t, what: str, dtype=torch.uint8):
+_Tensor, _U8, _I64 = torch.Tensor, torch.uint8, torch.int64
+
+
+def _dev_ptr(t, what: str, dtype=_U8):
     """Address of a contiguous tensor the kernels can dereference (or None):
     CUDA memory, or pinned host memory mapped into the device's address space
     (the kernels then read and write it over the CPU-GPU link; no copy).
     Pageable CPU tensors are refused: there is no CPU fallback."""
+    if type(t) is _Tensor and t.is_cuda and (t.dtype is dtype or dtype is None) and t.is_contiguous():
+        return t.data_ptr() if t.numel() else None  # the usual case, one look at each property
     if t is None:
         return None
     if not isinstance(t, torch.Tensor):
@@ -240,11 +245,19 @@ def _dev_ptr(t, what: str, dtype=torch.uint8):
     return t.data_ptr() if t.numel() > 0 else None
 
 
-def _stream_ptr(stream, device=None):
+# the current stream's handle of a device index, without the Stream object that
+# torch.cuda.current_stream() makes (0.1 against 2.4 us of a call's host time)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_ptr(stream, t=None):
+    """Handle of `stream` (a Stream or an int), or of the current stream of
+    tensor t's device (host tensors and t = None: the current device)."""
     if stream is None:
-        if device is not None and torch.device(device).type != "cuda":
-            device = None  # host (zero-copy) buffers: the current CUDA device
-        stream = torch.cuda.current_stream(device)
+        index = t.get_device() if t is not None else -1
+        if _raw_stream is not None and (index >= 0 or torch.cuda.is_initialized()):
+            return _raw_stream(index if index >= 0 else torch.cuda.current_device()) or None
+        stream = torch.cuda.current_stream(index if index >= 0 else None)
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
@@ -306,12 +319,14 @@ def stego_embed(cover, stego, msg, flags: int, result=None, geom=None, stream=No
     c = _dev_ptr(cover, "cover")
     s = _dev_ptr(stego, "stego")
     m = _dev_ptr(msg, "msg") if msg is not None else None
-    r = _dev_ptr(result, "result", torch.int64)
-    if stego.numel() != cover.numel():
+    r = _dev_ptr(result, "result", _I64) if result is not None else None
+    n = cover.numel()
+    if stego.numel() != n:
         raise ValueError("cover and stego sizes differ")
-    st = lib().stego_embed(c, s, cover.numel(), m, 0 if msg is None else msg.numel(),
-                           _geom(geom), int(flags), r, _stream_ptr(stream, cover.device))
-    _check(st, "stego_embed")
+    st = (_LIB or lib()).stego_embed(c, s, n, m, 0 if msg is None else msg.numel(), _geom(geom),
+                                     int(flags), r, _stream_ptr(stream, cover))
+    if st:
+        _check(st, "stego_embed")
 
 
 def stego_extract(stego, msg, msg_len: int, flags: int, result=None, geom=None,
@@ -320,11 +335,12 @@ def stego_extract(stego, msg, msg_len: int, flags: int, result=None, geom=None,
     ``result``; otherwise ``msg_len`` bytes are extracted."""
     s = _dev_ptr(stego, "stego")
     m = _dev_ptr(msg, "msg") if msg is not None else None
-    r = _dev_ptr(result, "result", torch.int64)
-    st = lib().stego_extract(s, stego.numel(), m, 0 if msg is None else msg.numel(),
-                             int(msg_len), _geom(geom), int(flags), r,
-                             _stream_ptr(stream, stego.device))
-    _check(st, "stego_extract")
+    r = _dev_ptr(result, "result", _I64) if result is not None else None
+    st = (_LIB or lib()).stego_extract(s, stego.numel(), m, 0 if msg is None else msg.numel(),
+                                       int(msg_len), _geom(geom), int(flags), r,
+                                       _stream_ptr(stream, stego))
+    if st:
+        _check(st, "stego_extract")
 
 
 def stego_extract_ballot(stego, msg, msg_len: int, flags: int, result=None, geom=None,
@@ -333,10 +349,10 @@ def stego_extract_ballot(stego, msg, msg_len: int, flags: int, result=None, geom
     layout only)."""
     s = _dev_ptr(stego, "stego")
     m = _dev_ptr(msg, "msg") if msg is not None else None
-    r = _dev_ptr(result, "result", torch.int64)
+    r = _dev_ptr(result, "result", _I64)
     st = lib().stego_extract_ballot(s, stego.numel(), m, 0 if msg is None else msg.numel(),
                                     int(msg_len), _geom(geom), int(flags), r,
-                                    _stream_ptr(stream, stego.device))
+                                    _stream_ptr(stream, stego))
     _check(st, "stego_extract_ballot")
 
 
@@ -345,8 +361,8 @@ def stego_changed_bytes(a, b, out2, stream=None) -> None:
     if a.numel() != b.numel():
         raise ValueError("sizes differ")
     st = lib().stego_changed_bytes(_dev_ptr(a, "a"), _dev_ptr(b, "b"), a.numel(),
-                                   _dev_ptr(out2, "out2", torch.int64),
-                                   _stream_ptr(stream, a.device))
+                                   _dev_ptr(out2, "out2", _I64),
+                                   _stream_ptr(stream, a))
     _check(st, "stego_changed_bytes")
 
 
@@ -356,19 +372,19 @@ def stego_batched_workspace_bytes(n: int) -> int:
 
 def stego_embed_batched(descs, n: int, results, flags: int, ws, tune=None, stream=None) -> None:
     st = lib().stego_embed_batched(_dev_ptr(descs, "descs", None), int(n),
-                                   _dev_ptr(results, "results", torch.int64), int(flags),
+                                   _dev_ptr(results, "results", _I64), int(flags),
                                    _tune(tune), _dev_ptr(ws, "ws", None),
                                    ws.numel() * ws.element_size(),
-                                   _stream_ptr(stream, descs.device))
+                                   _stream_ptr(stream, descs))
     _check(st, "stego_embed_batched")
 
 
 def stego_extract_batched(descs, n: int, results, flags: int, ws, tune=None, stream=None) -> None:
     st = lib().stego_extract_batched(_dev_ptr(descs, "descs", None), int(n),
-                                     _dev_ptr(results, "results", torch.int64), int(flags),
+                                     _dev_ptr(results, "results", _I64), int(flags),
                                      _tune(tune), _dev_ptr(ws, "ws", None),
                                      ws.numel() * ws.element_size(),
-                                     _stream_ptr(stream, descs.device))
+                                     _stream_ptr(stream, descs))
     _check(st, "stego_extract_batched")
 
 
@@ -383,8 +399,8 @@ def stego_embed_batched_noalloc(descs, n: int, results, flags: int, tune=None,
     for it.  At most NOALLOC_MAX_DESCS covers; calls that overlap on the GPU
     race on the shared scratch, so issue them on one stream."""
     st = lib().stego_embed_batched_noalloc(_dev_ptr(descs, "descs", None), int(n),
-                                           _dev_ptr(results, "results", torch.int64), int(flags),
-                                           _tune(tune), _stream_ptr(stream, descs.device))
+                                           _dev_ptr(results, "results", _I64), int(flags),
+                                           _tune(tune), _stream_ptr(stream, descs))
     _check(st, "stego_embed_batched_noalloc")
 
 
@@ -436,7 +452,7 @@ class BatchedGraph:
     def __init__(self, op: int, descs, n: int, results, flags: int, ws, tune=None):
         h = _vp(0)
         st = lib().stego_graph_capture_batched(int(op), _dev_ptr(descs, "descs", None), int(n),
-                                               _dev_ptr(results, "results", torch.int64),
+                                               _dev_ptr(results, "results", _I64),
                                                int(flags), _tune(tune), _dev_ptr(ws, "ws", None),
                                                ws.numel() * ws.element_size(), ctypes.byref(h))
         _check(st, "stego_graph_capture_batched")
