@@ -219,6 +219,15 @@ int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_s
     return (int)(want < cap ? want : cap);
 }
 
+int one_pass_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm, uint64_t units,
+                  uint64_t units_per_cta)
+{
+    if (ctas_per_sm > 0)
+        return persistent_grid(kernel, threads, smem, ctas_per_sm, units, units_per_cta);
+    const uint64_t want = (units + units_per_cta - 1) / units_per_cta;
+    return (int)(want < 1 ? 1 : want < (1u << 30) ? want : (1u << 30));
+}
+
 cudaError_t write_result(stego_result *res, uint64_t msg_bytes, int status, cudaStream_t s)
 {
     write_result_kernel<<<1, 1, 0, s>>>(res, msg_bytes, status);
@@ -377,8 +386,9 @@ int stego_embed(const uint8_t *d_cover, uint8_t *d_stego, uint64_t cover_bytes,
 
     cudaStream_t s = (cudaStream_t)stream;
     const Shape sh = shape_for(STEGO_OP_EMBED, nullptr);
-    // fused statistics: the stream's slot, or zeroed result fields
-    StatSlot *slot = stats ? stats_slot(s) : nullptr;
+    // the stream's slot (statistics, tile counter); statistics without one go
+    // into zeroed result fields
+    StatSlot *slot = stats_slot(s);
     if (stats && !slot && cudaMemsetAsync(d_result, 0, 2 * sizeof(uint64_t), s) != cudaSuccess)
         return STEGO_E_CUDA;
 

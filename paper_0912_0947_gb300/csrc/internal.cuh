@@ -54,6 +54,14 @@ unsigned long long context_id();
 int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm,
                     uint64_t units, uint64_t units_per_cta);
 
+// Grid of a kernel that reads and writes a little per CTA and adds nothing up: one
+// CTA per units_per_cta units, dealt out in order by the hardware, so that the
+// CTAs in flight work on one moving window of memory (a plain copy of 201 MB
+// back to back: 61 us, 66-68 us as a persistent grid whose CTAs drift apart),
+// unless the launch shape asks for a persistent grid (ctas_per_sm > 0).
+int one_pass_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm, uint64_t units,
+                  uint64_t units_per_cta);
+
 // Programmatic dependent launch: the kernel may be launched while the kernel
 // before it in the stream is still finishing (its CTAs then wait on the SMs
 // instead of behind the launch).  Only for kernels that call
@@ -82,16 +90,17 @@ __device__ __forceinline__ void allow_dependents()
 // Fused statistics without a zeroing copy
 // ---------------------------------------------------------------------------
 
-// Accumulator of one launch's changed-byte count and squared error, one per
-// stream (a static device array, zero at load).  Every CTA adds its partial
-// totals and then takes a ticket; the CTA with the last ticket moves the
-// totals into the result and clears the slot for the stream's next launch.
+// Accumulator of one launch's changed-byte count and squared error and its tile
+// counter, one per stream (a static device array, zero at load).  Every CTA
+// adds its partial totals and then takes a ticket; the CTA with the last
+// ticket moves the totals into the result and clears the slot for the stream's
+// next launch.
 struct StatSlot {
     unsigned long long changed;
     unsigned long long sse;
     unsigned int arrived;
-    unsigned int pad;
-    unsigned long long pad2;
+    unsigned int next; // tiles claimed beyond each CTA's first (for_tiles)
+    unsigned long long pad;
 };
 
 // The slot of stream s on the current device, or nullptr: then the caller
@@ -111,7 +120,8 @@ StatSlot *stats_slot(cudaStream_t s);
 // error of the launch.  `res` (nullable) receives msg_bytes = res_msg_bytes
 // and status STEGO_OK from block 0 of the launch; with `stats`, res->changed
 // and res->sse accumulate the changed-byte count and squared error and must
-// have been zeroed by the caller.
+// have been zeroed by the caller unless `slot` is given.  `slot` is the stream's
+// slot or nullptr, with or without statistics (the tile counter is there too).
 // ---------------------------------------------------------------------------
 
 // STREAM1 embed.  n_bytes: bytes written (C out of place, T in place).
@@ -263,6 +273,62 @@ __device__ __forceinline__ void block_stats(unsigned long long a, unsigned long 
             __threadfence();
             res->changed = atomicExch(&slot->changed, 0ull);
             res->sse = atomicExch(&slot->sse, 0ull);
+            atomicExch(&slot->next, 0u);
+            atomicExch(&slot->arrived, 0u);
+        }
+    }
+}
+
+// Whether tiles are claimed: with a slot, and more than four for each CTA (with
+// fewer the CTAs have no time to drift, and the barrier per tile costs more:
+// 25 MB at odd addresses 12.0 us, 13.3 claimed).
+__device__ __forceinline__ bool tiles_claimed(const StatSlot *slot, uint32_t ntiles)
+{
+    return slot && ntiles > 4u * gridDim.x;
+}
+
+// Calls body(tile) for this CTA's tiles of ntiles, all its threads together:
+// the tile of its own index, then the next one that no CTA has taken yet
+// (tiles_claimed), else every gridDim.x-th.  Taken in order the tiles in flight stay
+// one moving window of memory: dealt by the grid's stride the CTAs drift apart
+// (a plain copy of 201 MB back to back: 66-68 us by stride, 61 us as one CTA per
+// tile; but a CTA per tile adds its statistics for each, three atomics on one
+// address, 70 -> 78 us for the one-bit embed).  The next claim is in flight
+// while a tile is worked on.  After it every CTA calls block_stats or
+// tiles_done once.  It pays where a kernel does little but move data: the k-bit
+// and paper-layout units and the comparison of two arrays measured slower
+// (8192x8192x3: k = 2 77 -> 80 us, one channel of the paper's layout 31 -> 34,
+// comparison 58 -> 63).
+template <typename Body>
+__device__ __forceinline__ void for_tiles(StatSlot *slot, uint32_t ntiles, Body &&body)
+{
+    __shared__ uint32_t s_next[2];
+    const bool claims = tiles_claimed(slot, ntiles);
+    uint32_t i = 0;
+    for (uint32_t tile = blockIdx.x; tile < ntiles;) {
+        uint32_t next = tile + gridDim.x;
+        if (claims && threadIdx.x == 0)
+            next = gridDim.x + atomicAdd(&slot->next, 1u);
+        body(tile);
+        if (claims) {
+            if (threadIdx.x == 0)
+                s_next[i] = next;
+            __syncthreads(); // (two words: the next write is two barriers from this read)
+            next = s_next[i];
+            i ^= 1u;
+        }
+        tile = next;
+    }
+}
+
+// Clears the tile counter for the stream's next launch (kernels that do not
+// call block_stats).
+__device__ __forceinline__ void tiles_done(StatSlot *slot, uint32_t ntiles)
+{
+    if (tiles_claimed(slot, ntiles) && threadIdx.x == 0) {
+        __threadfence(); // this CTA's claims are done before its ticket
+        if (atomicAdd(&slot->arrived, 1u) == gridDim.x - 1) {
+            atomicExch(&slot->next, 0u);
             atomicExch(&slot->arrived, 0u);
         }
     }

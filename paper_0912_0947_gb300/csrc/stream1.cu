@@ -44,12 +44,11 @@ __device__ __forceinline__ void write_res(const EmbedArgs &e, bool stats)
     }
 }
 
-// Vector path (cover and stego 16-byte aligned), persistent grid.  Whole
-// rounds of V vectors per thread cover the vectors up to the last multiple
-// of the grid's round; the remainder is spread one vector per thread over
-// the whole grid, so every CTA ends within a fraction of a round of the
-// others (with rounds dealt whole, a quarter of the CTAs would run one round
-// longer on the 201 MB cover).
+// Vector path (cover and stego 16-byte aligned), persistent grid; a tile is one
+// round of V vectors per thread (two and four rounds per tile: 66.3 and 68.3 us
+// where this takes 65.6).  HBM-bound: 201 MB at full capacity back to back 70.1
+// us with tiles dealt by the grid's stride, 65.7 us claimed in order, 0.96 of
+// the measured copy rate.
 template <int V, bool STATS>
 __global__ void __launch_bounds__(512) embed_vec(EmbedArgs e)
 {
@@ -58,36 +57,38 @@ __global__ void __launch_bounds__(512) embed_vec(EmbedArgs e)
     unsigned long long changed = 0, sse = 0;
     write_res(e, STATS);
     const uint64_t nvec = e.a.n_bytes >> 4;
-    const uint64_t round = (uint64_t)gridDim.x * blockDim.x * V;
-    const uint64_t whole = nvec / round * round;
-    s1::embed_vec_range<V, STATS>(e.a, (uint64_t)blockIdx.x * blockDim.x * V + threadIdx.x,
-                                  whole, round, changed, sse);
-    s1::embed_vec_range<1, STATS>(e.a, whole + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
-                                  nvec, (uint64_t)gridDim.x * blockDim.x, changed, sse);
+    const uint32_t round = blockDim.x * V;
+    const uint32_t ntiles = (uint32_t)((nvec + round - 1) / round);
+    for_tiles(e.slot, ntiles, [&](uint32_t tile) {
+        const uint64_t v0 = (uint64_t)tile * round;
+        s1::embed_vec_range<V, STATS>(e.a, v0 + threadIdx.x, v0 + round < nvec ? v0 + round : nvec,
+                                      round, changed, sse);
+    });
     if (blockIdx.x == 0)
         s1::embed_tail<STATS>(e.a, changed, sse);
     if (STATS)
         block_stats(changed, sse, e.res, e.slot);
+    else
+        tiles_done(e.slot, ntiles);
 }
 
 // The h head bytes and the bytes after the nvb aligned vectors that follow
-// them (fewer than 32 in all), one per thread of the calling CTA.
+// them (fewer than 160 in all), one per thread of the calling CTA.
 template <bool STATS>
 __device__ __forceinline__ void head_tail(const s1::EmbedView &a, uint32_t h, uint64_t nvb,
                                           unsigned long long &changed, unsigned long long &sse)
 {
     const uint32_t tail = (uint32_t)(a.n_bytes - h - (nvb << 4));
-    if (threadIdx.x < h + tail) {
-        const uint64_t k = threadIdx.x < h ? (uint64_t)threadIdx.x
-                                           : h + (nvb << 4) + (threadIdx.x - h);
+    for (uint32_t t = threadIdx.x; t < h + tail; t += blockDim.x) {
+        const uint64_t k = t < h ? (uint64_t)t : h + (nvb << 4) + (t - h);
         const uint32_t sb = k < a.t_bytes ? s1::stream_byte(a, k >> 3) : 0u;
         s1::embed_one<STATS>(a, k, sb, changed, sse);
     }
 }
 
 // Cover and stego with the same misalignment: aligned vectors after h head
-// bytes, the stream cut at bit h % 8; block 0 does the head and the tail
-// (fewer than 32 bytes).  Requires n_bytes >= h.
+// bytes, the stream cut at bit h % 8; the last CTA does the head and the tail.
+// Requires n_bytes >= h.  Tiles as in embed_vec.
 template <int V, bool STATS>
 __global__ void __launch_bounds__(512) embed_shift(EmbedArgs e, uint32_t h)
 {
@@ -96,20 +97,26 @@ __global__ void __launch_bounds__(512) embed_shift(EmbedArgs e, uint32_t h)
     unsigned long long changed = 0, sse = 0;
     write_res(e, STATS);
     const uint64_t nvb = (e.a.n_bytes - h) >> 4;
-    s1::embed_shift_range<V, STATS>(e.a, h, (uint64_t)blockIdx.x * blockDim.x * V + threadIdx.x,
-                                    nvb, (uint64_t)gridDim.x * blockDim.x * V, changed, sse);
-    if (blockIdx.x == 0)
+    const uint32_t round = blockDim.x * V;
+    const uint32_t ntiles = (uint32_t)((nvb + round - 1) / round);
+    if (blockIdx.x == gridDim.x - 1)
         head_tail<STATS>(e.a, h, nvb, changed, sse);
+    for_tiles(e.slot, ntiles, [&](uint32_t tile) {
+        const uint64_t j0 = (uint64_t)tile * round;
+        s1::embed_shift_range<V, STATS>(e.a, h, j0 + threadIdx.x, j0 + round < nvb ? j0 + round : nvb,
+                                        round, changed, sse);
+    });
     if (STATS)
         block_stats(changed, sse, e.res, e.slot);
+    else
+        tiles_done(e.slot, ntiles);
 }
 
 // Cover and stego at different addresses mod 16, out of place: aligned
 // stego vectors after h head bytes, each from two aligned cover vectors
 // (cover + h is 4Q + b bytes past a 16-byte boundary), the grid's warps
-// taking blocks of 32*V consecutive stego vectors; block 0 does the head and
-// the tail (fewer than 32 bytes).
-// Requires n_bytes >= h.
+// taking blocks of 32*V consecutive stego vectors; the last CTA does
+// the head and the tail.  Requires n_bytes >= h.  Tiles as in embed_vec.
 template <int Q, int V, bool STATS>
 __global__ void __launch_bounds__(512) embed_funnel(EmbedArgs e, uint32_t h, uint32_t sel)
 {
@@ -118,13 +125,19 @@ __global__ void __launch_bounds__(512) embed_funnel(EmbedArgs e, uint32_t h, uin
     unsigned long long changed = 0, sse = 0;
     write_res(e, STATS);
     const uint64_t nvb = (e.a.n_bytes - h) >> 4;
-    s1::embed_funnel_warp<Q, STATS, V>(e.a, h, sel, 0, nvb,
-                                       ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                                       ((uint64_t)gridDim.x * blockDim.x) >> 5, changed, sse);
-    if (blockIdx.x == 0)
+    const uint32_t round = blockDim.x * V;
+    const uint32_t ntiles = (uint32_t)((nvb + round - 1) / round);
+    if (blockIdx.x == gridDim.x - 1)
         head_tail<STATS>(e.a, h, nvb, changed, sse);
+    for_tiles(e.slot, ntiles, [&](uint32_t tile) {
+        const uint64_t j0 = (uint64_t)tile * round;
+        s1::embed_funnel_warp<Q, STATS, V>(e.a, h, sel, j0, j0 + round < nvb ? j0 + round : nvb,
+                                           threadIdx.x >> 5, blockDim.x >> 5, changed, sse);
+    });
     if (STATS)
         block_stats(changed, sse, e.res, e.slot);
+    else
+        tiles_done(e.slot, ntiles);
 }
 
 // Byte path for cover and stego with different misalignments: one thread
@@ -149,15 +162,16 @@ using s1::extract_prologue;
 // Vector path: stego 16-byte aligned.  The first round's loads are issued
 // before the header is read (bounded by the longest message the call can
 // produce, so they stay inside the stego); the round is then written for the
-// header's length.  Later rounds: whole rounds, then the remainder spread
-// one vector per thread as in embed_vec.
+// header's length.  One round per CTA (see one_pass_grid; 201 MB back to back 36.5
+// -> 34.2 us, 0.97 of the measured copy rate); with a persistent grid whole
+// rounds follow, then the remainder spread one vector per thread.
 template <int V>
 __global__ void __launch_bounds__(512) extract_vec(ExtractArgs a)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
-    const uint64_t first = (uint64_t)blockIdx.x * blockDim.x * V + threadIdx.x;
-    const uint64_t round = (uint64_t)gridDim.x * blockDim.x * V;
+    const uint32_t round = blockDim.x * V;
+    const uint64_t first = (uint64_t)blockIdx.x * round + threadIdx.x;
     const uint4 *__restrict__ src =
         reinterpret_cast<const uint4 *>(a.st + (a.header ? 32u : 0u));
     uint4 c[V];
@@ -184,9 +198,10 @@ __global__ void __launch_bounds__(512) extract_vec(ExtractArgs a)
             x.msg[2 * v + 1] = (uint8_t)(pair >> 8);
         }
     }
-    const uint64_t whole = nvec / round * round;
-    s1::extract_vec_range<V>(x, first + round, whole, round);
-    const uint64_t rest = whole > round ? whole : round; // vectors below: done above
+    const uint64_t step = (uint64_t)gridDim.x * round; // (a launch shape with a persistent grid)
+    const uint64_t whole = nvec / step * step;
+    s1::extract_vec_range<V>(x, first + step, whole, step);
+    const uint64_t rest = whole > step ? whole : step; // vectors below: done above
     s1::extract_vec_range<1>(x, rest + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nvec,
                              (uint64_t)gridDim.x * blockDim.x);
     if ((x.len & 1u) && blockIdx.x == 0 && threadIdx.x == 0)
@@ -219,7 +234,9 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // 201 MB cover at full capacity (with the check-free interior rounds):
 // same misalignment embed 69.6 / 69.7 / 69.2 us for 1 / 2 / 4 (83-88 us
 // before those rounds), and with the message words' address computed once
-// per round 70.0-71.7 / 67.6-68.9 us for 2 / 4; different misalignments, both cover vectors loaded
+// per round 70.0-71.7 / 67.6-68.9 us for 2 / 4 (L2 flushed; back to back 71.7
+// by stride, 68.8 with tiles claimed in order, in place 75.3 -> 68.5);
+// different misalignments, both cover vectors loaded
 // per stego vector, 82.7 / 72.4-73.7 / 71.7-84.7 us, and with the second
 // vector shuffled from the next lane 71.7-74.5 us at 2 and 4 alike (4 kept:
 // the batched kernel shares the routine and gains there); extraction 48.7
@@ -230,6 +247,10 @@ constexpr int kFunnelV = 4;
 constexpr int kExtractShiftV = 4;
 
 int clamp_vec(int v) { return (v == 1 || v == 2 || v == 8) ? v : 4; }
+
+// Threads of the misaligned embeds' CTAs at most: 3839x2159x3, both 13 bytes
+// past a boundary, 12.1 us with 256, 13.7 with 512; 8192x8192x3 68.8 / 69.0.
+constexpr int kShiftThreads = 256;
 
 } // namespace
 
@@ -251,14 +272,13 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
     e.a.pad = 0;
     e.res = res;
     e.res_msg_bytes = res_msg_bytes;
-    e.slot = stats ? slot : nullptr;
-    const int T = sh.threads;
+    e.slot = slot;
     void *args[] = {&e};
     if (aligned16(cover) && aligned16(stego) && bulk_stages(sh))
         return s1_embed_bulk(cover, stego, n_bytes, t_bytes, msg, slen, header, nbits, stats,
                              res, res_msg_bytes, sh, s, slot);
     if (aligned16(cover) && aligned16(stego)) {
-        const int vec = clamp_vec(sh.vec);
+        const int vec = clamp_vec(sh.vec), T = sh.threads;
         const void *k = nullptr;
         switch (vec) {
         case 1: k = stats ? (const void *)embed_vec<1, true> : (const void *)embed_vec<1, false>; break;
@@ -271,7 +291,11 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
                                          (uint64_t)T * vec);
         return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
     }
-    const uint32_t h = (uint32_t)((16u - ((uintptr_t)cover & 15u)) & 15u);
+    // heads up to a 128-byte boundary of the stego, so that a warp's vectors are
+    // whole cache lines (16-byte boundaries in a small cover)
+    const int T = sh.threads < kShiftThreads ? sh.threads : kShiftThreads;
+    const uint32_t line = n_bytes >= 16384u ? 127u : 15u;
+    const uint32_t h = (uint32_t)(-(uintptr_t)cover & line);
     if ((((uintptr_t)cover ^ (uintptr_t)stego) & 15u) == 0 && n_bytes >= (uint64_t)h + 16u) {
         const void *k = stats ? (const void *)embed_shift<kShiftV, true>
                               : (const void *)embed_shift<kShiftV, false>;
@@ -280,7 +304,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         void *sargs[] = {&e, (void *)&h};
         return launch_dependent(k, dim3(grid), dim3(T), sargs, 0, s);
     }
-    const uint32_t hs = (uint32_t)((16u - ((uintptr_t)stego & 15u)) & 15u);
+    const uint32_t hs = (uint32_t)(-(uintptr_t)stego & line);
     if (cover != stego && n_bytes >= (uint64_t)hs + 16u) {
         const uint32_t d = (uint32_t)(((uintptr_t)cover + hs) & 15u), b = d & 3u;
         const uint32_t sel = b | ((b + 1) << 4) | ((b + 2) << 8) | ((b + 3) << 12);
@@ -337,7 +361,7 @@ cudaError_t s1_extract(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_t cap
         default: k = (const void *)extract_vec<4>; break;
         }
         const uint64_t nvec = max_len >> 1;
-        const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvec > 0 ? nvec : 1,
+        const int grid = one_pass_grid(k, T, 0, sh.ctas_per_sm, nvec > 0 ? nvec : 1,
                                          (uint64_t)T * vec);
         return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
     }
