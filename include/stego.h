@@ -51,7 +51,8 @@
  *     case the message buffer is not written.  STEGO_E_CUDA means a CUDA
  *     launch or memset failed (see cudaGetLastError in the caller's runtime).
  *   - Any byte alignment is accepted.  Cover and stego buffers that start on
- *     16-byte boundaries take the vectorised (128-bit) path.
+ *     16-byte boundaries take the shortest path; all others run in whole
+ *     vectors too, joined from the aligned ones around them.
  *   - In-place embedding (d_stego == d_cover) is allowed and then bytes past
  *     the embedded bits are not written.  Any other overlap between the
  *     buffers of one call is STEGO_E_INVAL.
@@ -283,8 +284,9 @@ uint64_t stego_batched_workspace_bytes(uint32_t n);
  *              scratch: its contents on entry do not matter and on return
  *              are unspecified.
  * Both layouts may be mixed in one batch.  One-bit stream covers are cut
- * into tiles of cover bytes; paper-layout covers into tiles of whole rows
- * (out of place: rows are copied, then their plane bytes rewritten).
+ * into tiles of cover bytes; paper-layout covers into tiles of 16-pixel units
+ * (1, 3 or 4 channels) or of whole rows (rows copied, then their plane bytes
+ * rewritten).
  * Descriptor errors (capacity, geometry, overlap) are per cover: that
  * cover's status is set and its output is not written; other covers
  * proceed.  Returns STEGO_E_NOMEM when ws_bytes is too small. */
@@ -324,7 +326,7 @@ int stego_embed_batched_noalloc(const stego_desc *d_descs, uint32_t n, stego_res
 
 /* CUDA graph of one batched call.  The descriptors, results and workspace
  * are captured by address: fill the same device arrays with new descriptors
- * (same n) and replay, which re-runs the three launches of the call without
+ * (same n) and replay, which re-runs the launches of the call without
  * host-side launch overhead.  The graph object (and its instantiation) is
  * the only thing these functions create; stego_graph_destroy releases it.
  *   op  STEGO_OP_EMBED_BATCHED or STEGO_OP_EXTRACT_BATCHED.

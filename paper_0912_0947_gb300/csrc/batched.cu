@@ -24,10 +24,10 @@
 //                           the scan)
 //   [info_off, +64n)        per-descriptor derived sizes, geometry and mode
 // Both layouts batch: the one-bit stream in tiles of cover bytes; the
-// paper's layout (Sections VI/VII) in tiles of whole rows (copy, barrier,
-// scatter out of place; scatter in place) and, for extraction, of 16-byte
-// message runs (1, 3 or 4 channels) or rows, with the routines the
-// single-image kernels use.  The paper layout has its own persistent
+// paper's layout (Sections VI/VII) in tiles of 16-pixel units (1, 3 or 4
+// channels) or of whole rows (copy, barrier, scatter out of place; scatter in
+// place) and, for extraction, of 16-byte message runs or rows, with the
+// routines the single-image kernels use.  The paper layout has its own persistent
 // kernels (own tile offsets and counter), so its register needs do not
 // touch the stream kernels'.
 #include <cooperative_groups.h>
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(kMisExtractThreads)
 // with two, although it spills; extract 381 against 410).  One unit or run at a
 // time: with four CTAs the warps hide the latency, and two in flight were
 // slower.  With rows that are not whole vectors copied and then scattered byte
-// by byte the same batch took 2824 us (embed) and 505 us (extract), now 900
+// by byte the same batch took 2823 us (embed) and 505 us (extract), now 900
 // and 395; large RGB covers run at 0.75 of the copy rate, gray ones, with
 // three times the units per byte, at 0.53.
 template <bool STATS>

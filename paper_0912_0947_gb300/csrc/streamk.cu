@@ -670,7 +670,7 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t ulo, uin
 #pragma unroll
         for (int r = 0; r < U; ++r) {
             const uint64_t u = u0 + (uint64_t)r * blockDim.x;
-            if (u < nunits && u >= ulo) {
+            if (u < nunits && (!FLAT || u >= ulo)) {
                 read_unit<CH, FLAT>(a, u, w[r]);
             } else {
 #pragma unroll
@@ -696,7 +696,7 @@ __device__ __forceinline__ void extract3_units(const KView &a, uint64_t ulo, uin
                     op[0] = P;
                     op[1] = __byte_perm(Q, Pn, 0x5410u);
                 }
-            } else if (u < nunits && u >= ulo) {
+            } else if (u < nunits && (!FLAT || u >= ulo)) {
                 const uint64_t q0 = 6u * u; // first stream byte of the unit
                 if (q0 >= hb && q0 + 6 <= sbytes && ((q0 - hb + (uintptr_t)a.out) & 1u) == 0) {
                     unsigned short *op = reinterpret_cast<unsigned short *>(a.out + (q0 - hb));
@@ -760,13 +760,13 @@ __global__ void __launch_bounds__(512) extractk_units(KView a)
 #pragma unroll
         for (int r = 0; r < U; ++r) {
             const uint64_t u = v0 + (uint64_t)r * blockDim.x;
-            if (u < nunits && u >= ulo)
+            if (u < nunits && (!FLAT || u >= ulo))
                 read_unit<CH, FLAT>(a, u, w[r]);
         }
 #pragma unroll
         for (int r = 0; r < U; ++r) {
             const uint64_t u = v0 + (uint64_t)r * blockDim.x;
-            if (u >= nunits || u < ulo)
+            if (u >= nunits || (FLAT && u < ulo))
                 continue;
             uint32_t g[4];
             get_unit<CH>(w[r], a.f.sel, g);
