@@ -558,12 +558,14 @@ __device__ __forceinline__ uint32_t claim_size(unsigned long long left)
 
 // Tiles of a small batch are cut in 2^shift parts (down to 4096 bytes), until
 // every CTA has a few or they are no smaller than that: 16 covers of sides 64
-// to 512 are 50 tiles of 64 KiB, which 50 CTAs took one after another.
+// to 512 are 50 tiles of 64 KiB, which 50 CTAs took one after another.  A part
+// is a whole number of 16-byte vectors, so that the parts of tile_bytes (and of
+// a misaligned tile's tile_bytes / 16 vectors or byte pairs) make up the tile.
 __device__ __forceinline__ uint32_t split_shift(unsigned long long total, uint32_t tile_bytes)
 {
     uint32_t s = 0;
     while (total << s < 2ull * gridDim.x && (tile_bytes >> (s + 1)) >= 4096u &&
-           (tile_bytes & ((2u << s) - 1u)) == 0u)
+           (tile_bytes & ((32u << s) - 1u)) == 0u)
         ++s;
     return s;
 }
@@ -859,7 +861,7 @@ __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescIn
         a.pad = 0;
         const uint32_t h = inf.W;
         const uint64_t nvb = (inf.n_bytes - h) >> 4;
-        // (a misaligned tile is tile_bytes / 16 vectors: whole parts)
+        // (a misaligned tile is tile_bytes / 16 vectors: whole parts, see split_shift)
         const uint64_t per = inf.per_tile >> shift;
         const uint64_t j0 = lt * per, je = j0 + (uint64_t)cnt * per;
         const uint64_t j1 = je < nvb ? je : nvb;
