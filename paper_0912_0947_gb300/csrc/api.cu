@@ -219,13 +219,10 @@ int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_s
     return (int)(want < cap ? want : cap);
 }
 
-int one_pass_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm, uint64_t units,
-                  uint64_t units_per_cta)
+int one_pass_grid(uint64_t units, uint64_t units_per_cta)
 {
-    if (ctas_per_sm > 0)
-        return persistent_grid(kernel, threads, smem, ctas_per_sm, units, units_per_cta);
     const uint64_t want = (units + units_per_cta - 1) / units_per_cta;
-    return (int)(want < 1 ? 1 : want < (1u << 30) ? want : (1u << 30));
+    return (int)(want < 1 ? 1 : want < 0x7FFFFFFFull ? want : 0x7FFFFFFFull);
 }
 
 cudaError_t write_result(stego_result *res, uint64_t msg_bytes, int status, cudaStream_t s)

@@ -54,13 +54,13 @@ unsigned long long context_id();
 int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm,
                     uint64_t units, uint64_t units_per_cta);
 
-// Grid of a kernel that reads and writes a little per CTA and adds nothing up: one
-// CTA per units_per_cta units, dealt out in order by the hardware, so that the
-// CTAs in flight work on one moving window of memory (a plain copy of 201 MB
-// back to back: 61 us, 66-68 us as a persistent grid whose CTAs drift apart),
-// unless the launch shape asks for a persistent grid (ctas_per_sm > 0).
-int one_pass_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm, uint64_t units,
-                  uint64_t units_per_cta);
+// Grid of a kernel that does units_per_cta units per CTA, however many CTAs these
+// make (fewer than 2^31), and adds nothing up: dealt out in order by the hardware,
+// the CTAs in flight work on one moving window of memory (a plain copy of 201 MB
+// back to back: 61 us, 66-68 us as a persistent grid whose CTAs drift apart).  Only
+// where the work is known when the kernel is launched: CTAs that find nothing to do
+// cost some 2.5 us for each wave of them.
+int one_pass_grid(uint64_t units, uint64_t units_per_cta);
 
 // Programmatic dependent launch: the kernel may be launched while the kernel
 // before it in the stream is still finishing (its CTAs then wait on the SMs

@@ -159,21 +159,29 @@ __global__ void __launch_bounds__(512) embed_bytes(EmbedArgs e)
 using s1::ExtractArgs;
 using s1::extract_prologue;
 
-// Vector path: stego 16-byte aligned.  The first round's loads are issued
-// before the header is read (bounded by the longest message the call can
-// produce, so they stay inside the stego); the round is then written for the
-// header's length.  One round per CTA (see one_pass_grid; 201 MB back to back 36.5
-// -> 34.2 us, 0.97 of the measured copy rate); with a persistent grid whole
-// rounds follow, then the remainder spread one vector per thread.
+// Message byte pair v.
+__device__ __forceinline__ void put_pair(const ExtractView &x, uint64_t v, uint32_t pair)
+{
+    if (x.msg_even) {
+        *reinterpret_cast<unsigned short *>(x.msg + 2 * v) = (unsigned short)pair;
+    } else {
+        x.msg[2 * v] = (uint8_t)pair;
+        x.msg[2 * v + 1] = (uint8_t)(pair >> 8);
+    }
+}
+
+// Stego 16-byte aligned, the length known to the caller: one round of V vectors
+// per thread and CTA, the CTAs dealt out in memory order (see one_pass_grid; 201
+// MB back to back 35.5 us on a persistent grid, 33.5 so, 0.99 of the measured
+// copy rate).
 template <int V>
-__global__ void __launch_bounds__(512) extract_vec(ExtractArgs a)
+__global__ void __launch_bounds__(512) extract_once(ExtractArgs a)
 {
     grid_dependency_wait(); // launched dependent: nothing is touched before
     allow_dependents();
-    const uint32_t round = blockDim.x * V;
-    const uint64_t first = (uint64_t)blockIdx.x * round + threadIdx.x;
-    const uint4 *__restrict__ src =
-        reinterpret_cast<const uint4 *>(a.st + (a.header ? 32u : 0u));
+    ExtractView x;
+    const uint64_t first = (uint64_t)blockIdx.x * blockDim.x * V + threadIdx.x;
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.st);
     uint4 c[V];
 #pragma unroll
     for (int u = 0; u < V; ++u) {
@@ -181,31 +189,78 @@ __global__ void __launch_bounds__(512) extract_vec(ExtractArgs a)
         if (v < a.max_vec)
             c[u] = __ldcs(src + v);
     }
+    extract_prologue(a, x);
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        const uint64_t v = first + (uint64_t)u * blockDim.x;
+        if (v < a.max_vec)
+            put_pair(x, v, s1::gather16(c[u]));
+    }
+    if ((x.len & 1u) && blockIdx.x == 0 && threadIdx.x == 0)
+        s1::extract_one(x, x.len - 1);
+}
+
+// Stego 16-byte aligned, the length in its header (or a launch shape with a
+// persistent grid): each warp takes rounds of 32*V consecutive vectors by the
+// grid's stride.  The first round's loads are issued before the header is read,
+// bounded by the longest message the call can produce, so that they stay inside
+// the stego; the grid is one wave of CTAs, so that they are no more than some 15
+// MB however much longer the buffer is than the message.  A CTA per round for the
+// whole capacity loads all of it ahead of the header, and reading the header first
+// in the CTAs after the first wave still leaves them to be launched: 201 MB, 1 KB
+// message, capacity-sized buffer 30.9 and 25.7 us, this 3.2; at full capacity
+// 34.3 and 37.8, this 35.1 (36.5 with rounds of a CTA in place of a warp's; rounds
+// claimed from a counter 37-117); 786 KB 1.9.  The registers are bounded for the warps per SM
+// of the loads in flight (V = 4: twelve CTAs of 128 threads; at 64 registers 36.4).
+template <int V>
+__global__ void __launch_bounds__(512, V >= 8 ? 2 : V == 4 ? 3 : 4) extract_vec(ExtractArgs a)
+{
+    grid_dependency_wait(); // launched dependent: nothing is touched before
+    allow_dependents();
+    constexpr uint32_t round = 32u * V;
+    const uint32_t lane = threadIdx.x & 31u, wpb = blockDim.x >> 5;
+    const uint64_t step = (uint64_t)gridDim.x * wpb * round;
+    const uint4 *__restrict__ src =
+        reinterpret_cast<const uint4 *>(a.st + (a.header ? 32u : 0u));
+    uint64_t v0 = ((uint64_t)blockIdx.x * wpb + (threadIdx.x >> 5)) * round + lane;
+    uint4 c[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u)
+        if (v0 + 32u * u < a.max_vec)
+            c[u] = __ldcs(src + v0 + 32u * u);
     ExtractView x;
     if (extract_prologue(a, x) != STEGO_OK)
         return;
     const uint64_t nvec = x.len >> 1;
+    for (bool loaded = true; v0 - lane < nvec; v0 += step, loaded = false) {
+        if (v0 - lane + round <= nvec) {
+            if (!loaded) {
 #pragma unroll
-    for (int u = 0; u < V; ++u) {
-        const uint64_t v = first + (uint64_t)u * blockDim.x;
-        if (v >= nvec)
-            continue;
-        const uint32_t pair = s1::gather16(c[u]);
-        if (x.msg_even) {
-            *reinterpret_cast<unsigned short *>(x.msg + 2 * v) = (unsigned short)pair;
-        } else {
-            x.msg[2 * v] = (uint8_t)pair;
-            x.msg[2 * v + 1] = (uint8_t)(pair >> 8);
+                for (int u = 0; u < V; ++u)
+                    c[u] = __ldcs(src + v0 + 32u * u);
+            }
+#pragma unroll
+            for (int u = 0; u < V; ++u)
+                put_pair(x, v0 + 32u * u, s1::gather16(c[u]));
+        } else { // the message ends in this round
+#pragma unroll
+            for (int u = 0; u < V; ++u)
+                if (!loaded && v0 + 32u * u < nvec)
+                    c[u] = __ldcs(src + v0 + 32u * u);
+#pragma unroll
+            for (int u = 0; u < V; ++u)
+                if (v0 + 32u * u < nvec)
+                    put_pair(x, v0 + 32u * u, s1::gather16(c[u]));
         }
     }
-    const uint64_t step = (uint64_t)gridDim.x * round; // (a launch shape with a persistent grid)
-    const uint64_t whole = nvec / step * step;
-    s1::extract_vec_range<V>(x, first + step, whole, step);
-    const uint64_t rest = whole > step ? whole : step; // vectors below: done above
-    s1::extract_vec_range<1>(x, rest + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nvec,
-                             (uint64_t)gridDim.x * blockDim.x);
     if ((x.len & 1u) && blockIdx.x == 0 && threadIdx.x == 0)
         s1::extract_one(x, x.len - 1);
+}
+
+template <int V>
+const void *extract_kernel(bool once)
+{
+    return once ? (const void *)extract_once<V> : (const void *)extract_vec<V>;
 }
 
 // A stego that is not 16-byte aligned: the warps of the grid take rounds
@@ -353,16 +408,17 @@ cudaError_t s1_extract(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_t cap
         return s1_extract_bulk(st, C, msg, cap, raw_len, header, res, sh, s);
     if (aligned16(st)) {
         const int vec = clamp_vec(sh.vec);
+        const bool once = !header && sh.ctas_per_sm == 0;
         const void *k;
         switch (vec) {
-        case 1: k = (const void *)extract_vec<1>; break;
-        case 2: k = (const void *)extract_vec<2>; break;
-        case 8: k = (const void *)extract_vec<8>; break;
-        default: k = (const void *)extract_vec<4>; break;
+        case 1: k = extract_kernel<1>(once); break;
+        case 2: k = extract_kernel<2>(once); break;
+        case 8: k = extract_kernel<8>(once); break;
+        default: k = extract_kernel<4>(once); break;
         }
-        const uint64_t nvec = max_len >> 1;
-        const int grid = one_pass_grid(k, T, 0, sh.ctas_per_sm, nvec > 0 ? nvec : 1,
-                                         (uint64_t)T * vec);
+        const uint64_t nvec = max_len >> 1, per_cta = (uint64_t)T * vec;
+        const int grid = once ? one_pass_grid(nvec, per_cta)
+                              : persistent_grid(k, T, 0, sh.ctas_per_sm, nvec, per_cta);
         return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
     }
     const void *k = (const void *)extract_shift<kExtractShiftV>;
