@@ -206,6 +206,15 @@ cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, void **a
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
+cudaError_t launch_counting(const void *kernel, dim3 grid, dim3 block, void **args, size_t smem,
+                            cudaStream_t s, void *totals, const StatSlot *slot)
+{
+    if (!totals || slot)
+        return launch_dependent(kernel, grid, block, args, smem, s);
+    const cudaError_t e = cudaMemsetAsync(totals, 0, 2 * sizeof(uint64_t), s);
+    return e != cudaSuccess ? e : cudaLaunchKernel(kernel, grid, block, args, smem, s);
+}
+
 int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_sm,
                     uint64_t units, uint64_t units_per_cta)
 {
@@ -383,11 +392,7 @@ int stego_embed(const uint8_t *d_cover, uint8_t *d_stego, uint64_t cover_bytes,
 
     cudaStream_t s = (cudaStream_t)stream;
     const Shape sh = shape_for(STEGO_OP_EMBED, nullptr);
-    // the stream's slot (statistics, tile counter); statistics without one go
-    // into zeroed result fields
-    StatSlot *slot = stats_slot(s);
-    if (stats && !slot && cudaMemsetAsync(d_result, 0, 2 * sizeof(uint64_t), s) != cudaSuccess)
-        return STEGO_E_CUDA;
+    StatSlot *slot = stats_slot(s); // statistics, tile counter
 
     if (layout == STEGO_LAYOUT_STREAM1 && (k != 1 || plane_only)) {
         if (cover_bytes == 0 || (!header && msg_bytes == 0 && inplace)) {
@@ -544,12 +549,9 @@ int stego_changed_bytes(const uint8_t *d_a, const uint8_t *d_b, uint64_t n, uint
     if (overlap(d_out2, 2 * sizeof(uint64_t), d_a, n) || overlap(d_out2, 2 * sizeof(uint64_t), d_b, n))
         return STEGO_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    // the totals go through the stream's slot, or into zeroed words
-    StatSlot *slot = n ? stats_slot(s) : nullptr;
-    if (!slot && cudaMemsetAsync(d_out2, 0, 2 * sizeof(uint64_t), s) != cudaSuccess)
-        return STEGO_E_CUDA;
     if (n == 0)
-        return STEGO_OK;
+        return cuda_status(cudaMemsetAsync(d_out2, 0, 2 * sizeof(uint64_t), s));
+    StatSlot *slot = stats_slot(s);
     const Shape sh = shape_for(STEGO_OP_CHANGED, nullptr);
     return cuda_status(changed_bytes(d_a, d_b, n, reinterpret_cast<unsigned long long *>(d_out2), sh, s, slot));
 }

@@ -547,7 +547,7 @@ cudaError_t s1_embed_bulk(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes
     const uint64_t ntiles = ((n_bytes >> 4) + tvec - 1) / tvec;
     const int grid = persistent_grid(k, sh.threads, ring, sh.ctas_per_sm, ntiles ? ntiles : 1, 1);
     void *args[] = {&e};
-    return launch_dependent(k, dim3(grid), dim3(sh.threads), args, ring, s);
+    return launch_counting(k, dim3(grid), dim3(sh.threads), args, ring, s, stats ? res : nullptr, slot);
 }
 
 cudaError_t s1_extract_bulk(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_t cap,

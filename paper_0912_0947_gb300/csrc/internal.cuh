@@ -62,6 +62,8 @@ int persistent_grid(const void *kernel, int threads, size_t smem, int ctas_per_s
 // cost some 2.5 us for each wave of them.
 int one_pass_grid(uint64_t units, uint64_t units_per_cta);
 
+struct StatSlot;
+
 // Programmatic dependent launch: the kernel may be launched while the kernel
 // before it in the stream is still finishing (its CTAs then wait on the SMs
 // instead of behind the launch).  Only for kernels that call
@@ -69,6 +71,16 @@ int one_pass_grid(uint64_t units, uint64_t units_per_cta);
 // cluster > 1: CTAs per thread block cluster (the grid a multiple of it).
 cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, void **args,
                              size_t smem, cudaStream_t s, uint32_t cluster = 1);
+
+// Launch of a kernel that adds to the two totals at `totals` (nullptr: a kernel
+// that does not, launched as a dependent): through the stream's slot, as a dependent
+// too; without one the totals are zeroed first, and the kernel is then an ordinary
+// launch.  (A dependent behind a memset was in a queue of 300 streams that stopped,
+// each a 256 MB copy, a memset and a dependent of 256 CTAs.  It was not found to be
+// the cause; CTAs that wait on the SMs for something other than a kernel
+// are the one thing that set that queue apart, and they are not needed.)
+cudaError_t launch_counting(const void *kernel, dim3 grid, dim3 block, void **args, size_t smem,
+                            cudaStream_t s, void *totals, const StatSlot *slot);
 
 // Returns once the grid before this one in the stream has completed and its
 // memory operations are visible (at once when there is none, or when the
@@ -119,9 +131,9 @@ StatSlot *stats_slot(cudaStream_t s);
 // Launchers (all stream-ordered, no synchronisation).  They return the CUDA
 // error of the launch.  `res` (nullable) receives msg_bytes = res_msg_bytes
 // and status STEGO_OK from block 0 of the launch; with `stats`, res->changed
-// and res->sse accumulate the changed-byte count and squared error and must
-// have been zeroed by the caller unless `slot` is given.  `slot` is the stream's
-// slot or nullptr, with or without statistics (the tile counter is there too).
+// and res->sse accumulate the changed-byte count and squared error (see
+// launch_counting).  `slot` is the stream's slot or nullptr, with or without
+// statistics (the tile counter is there too).
 // ---------------------------------------------------------------------------
 
 // STREAM1 embed.  n_bytes: bytes written (C out of place, T in place).
@@ -185,8 +197,7 @@ cudaError_t s1_extract_bulk(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_
                             uint64_t raw_len, bool header, stego_result *res, const Shape &sh,
                             cudaStream_t s);
 
-// Changed-byte count and SSE of two arrays into out2[0..1] (through the
-// stream's slot; without one they have been zeroed by the caller).
+// Changed-byte count and SSE of two arrays into out2[0..1].
 cudaError_t changed_bytes(const uint8_t *a, const uint8_t *b, uint64_t n,
                           unsigned long long *out2, const Shape &sh, cudaStream_t s,
                           StatSlot *slot);

@@ -184,12 +184,13 @@ const void *extract_units_kernel(uint32_t ch)
 } // namespace
 
 // Launches the unit kernel over a.f's units.
-static cudaError_t launch_units(const void *k, P2Args &a, uint32_t channels, cudaStream_t s)
+static cudaError_t launch_units(const void *k, P2Args &a, uint32_t channels, bool stats,
+                                cudaStream_t s)
 {
     const int grid = persistent_grid(k, kUnitThreads, 0, kAnyCtas, a.f.nunits,
                                      (uint64_t)kUnitThreads * units_per_thread(channels));
     void *args[] = {&a};
-    return launch_dependent(k, dim3(grid), dim3(kUnitThreads), args, 0, s);
+    return launch_counting(k, dim3(grid), dim3(kUnitThreads), args, 0, s, stats ? a.res : nullptr, a.slot);
 }
 
 bool p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
@@ -208,7 +209,7 @@ bool p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
     else
         k = stats ? units_kernel<true, false, false>(g.channels)
                   : units_kernel<false, false, false>(g.channels);
-    *err = launch_units(k, a, g.channels, s);
+    *err = launch_units(k, a, g.channels, stats, s);
     return true;
 }
 
@@ -225,12 +226,12 @@ cudaError_t p2_embed(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
         // kernel): whole vectors instead of one byte access per plane byte
         const void *k = stats ? units_kernel<true, true, false>(g.channels)
                               : units_kernel<false, true, false>(g.channels);
-        return launch_units(k, a, g.channels, s);
+        return launch_units(k, a, g.channels, stats, s);
     }
     const void *k = stats ? (const void *)p2_embed_rows<true> : (const void *)p2_embed_rows<false>;
     const int grid = row_grid(k, sh, a.v.R);
     void *args[] = {&a};
-    return launch_dependent(k, dim3(grid), dim3(sh.threads), args, 0, s);
+    return launch_counting(k, dim3(grid), dim3(sh.threads), args, 0, s, stats ? res : nullptr, slot);
 }
 
 cudaError_t p2_extract(const uint8_t *st, const stego_geom &g, uint8_t *msg, uint64_t N,

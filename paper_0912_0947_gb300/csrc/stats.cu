@@ -187,11 +187,11 @@ cudaError_t changed_bytes(const uint8_t *a, const uint8_t *b, uint64_t n,
         const uint4 *av = reinterpret_cast<const uint4 *>(a);
         const uint4 *bv = reinterpret_cast<const uint4 *>(b);
         void *args[] = {&av, &bv, (void *)&nvec, &a, &b, &n, &out2, &slot};
-        return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
+        return launch_counting(k, dim3(grid), dim3(T), args, 0, s, out2, slot);
     }
     if (n <= kBytesMost) {
         void *args[] = {&a, &b, &n, &out2, &slot};
-        return launch_dependent((const void *)changed_bytes_kernel, dim3(1), dim3(T), args, 0, s);
+        return launch_counting((const void *)changed_bytes_kernel, dim3(1), dim3(T), args, 0, s, out2, slot);
     }
     // from byte h on a's vectors and the vectors around b's bytes lie inside
     // the arrays (n > kBytesMost leaves room for h and a vector more)
@@ -210,7 +210,7 @@ cudaError_t changed_bytes(const uint8_t *a, const uint8_t *b, uint64_t n,
     }
     const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvec, (uint64_t)T * kShiftV);
     void *args[] = {&a, &b, &n, &h, (void *)&d, (void *)&nvec, &out2, &slot};
-    return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
+    return launch_counting(k, dim3(grid), dim3(T), args, 0, s, out2, slot);
 }
 
 } // namespace stego

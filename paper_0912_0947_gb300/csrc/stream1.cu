@@ -344,7 +344,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvec = n_bytes >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvec > 0 ? nvec : 1,
                                          (uint64_t)T * vec);
-        return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
+        return launch_counting(k, dim3(grid), dim3(T), args, 0, s, stats ? res : nullptr, slot);
     }
     // heads up to a 128-byte boundary of the stego, so that a warp's vectors are
     // whole cache lines (16-byte boundaries in a small cover)
@@ -357,7 +357,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvb = (n_bytes - h) >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvb, (uint64_t)T * kShiftV);
         void *sargs[] = {&e, (void *)&h};
-        return launch_dependent(k, dim3(grid), dim3(T), sargs, 0, s);
+        return launch_counting(k, dim3(grid), dim3(T), sargs, 0, s, stats ? res : nullptr, slot);
     }
     const uint32_t hs = (uint32_t)(-(uintptr_t)stego & line);
     if (cover != stego && n_bytes >= (uint64_t)hs + 16u) {
@@ -374,12 +374,12 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvb = (n_bytes - hs) >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvb, (uint64_t)T * F);
         void *fargs[] = {&e, (void *)&hs, (void *)&sel};
-        return launch_dependent(k, dim3(grid), dim3(T), fargs, 0, s);
+        return launch_counting(k, dim3(grid), dim3(T), fargs, 0, s, stats ? res : nullptr, slot);
     }
     const void *k = stats ? (const void *)embed_bytes<true> : (const void *)embed_bytes<false>;
     const uint64_t units = (n_bytes + 7) >> 3;
     const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, units > 0 ? units : 1, (uint64_t)T);
-    return launch_dependent(k, dim3(grid), dim3(T), args, 0, s);
+    return launch_counting(k, dim3(grid), dim3(T), args, 0, s, stats ? res : nullptr, slot);
 }
 
 cudaError_t s1_extract(const uint8_t *st, uint64_t C, uint8_t *msg, uint64_t cap,

@@ -936,7 +936,7 @@ cudaError_t sk_embed(const uint8_t *cover, uint8_t *stego, uint64_t C, uint32_t 
         const int TU = a.channels == 1 ? T : kAsyncThreads; // plane units: the pipeline's CTAs
         const int grid = persistent_grid(kern, TU, 0, kAnyCtas, a.f.nunits ? a.f.nunits : 1,
                                          (uint64_t)TU);
-        return launch_dependent(kern, dim3(grid), dim3(TU), args, 0, s);
+        return launch_counting(kern, dim3(grid), dim3(TU), args, 0, s, stats ? res : nullptr, slot);
     }
     if (plane_only && !inplace) {
         // the non-carrying bytes come from a copy of the cover (a stream
@@ -949,7 +949,7 @@ cudaError_t sk_embed(const uint8_t *cover, uint8_t *stego, uint64_t C, uint32_t 
     const void *kern = stats ? (const void *)embedk_bytes<true> : (const void *)embedk_bytes<false>;
     const int grid = persistent_grid(kern, T, 0, kAnyCtas, a.n_carry ? a.n_carry : 1,
                                      (uint64_t)T * 16);
-    return launch_dependent(kern, dim3(grid), dim3(T), args, 0, s);
+    return launch_counting(kern, dim3(grid), dim3(T), args, 0, s, stats ? res : nullptr, slot);
 }
 
 cudaError_t sk_extract(const uint8_t *st, uint64_t C, uint32_t k, bool plane_only,

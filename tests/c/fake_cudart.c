@@ -78,6 +78,11 @@ cudaError_t __cudaLaunchKernel(void *k, dim3 g, dim3 b, void **a, size_t m, void
     return cudaSuccess;
 }
 
+cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3 b, void **a, size_t m, cudaStream_t s)
+{
+    return __cudaLaunchKernel((void *)f, g, b, a, m, s);
+}
+
 /* -- the calls of the single-cover and batched entry points ------------------ */
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **a)
 {

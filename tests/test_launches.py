@@ -1,4 +1,6 @@
 """What a call queues, on a runtime that runs nothing (tests/launch_util.py)."""
+import ctypes
+
 import pytest
 
 import paper_0912_0947_gb300 as S
@@ -33,3 +35,47 @@ def test_known_length_extract_is_dealt_in_order(L):
     assert "extract_once" in name and grid == -(-(C // 16) // (4 * block))
     q = L.queued("stego_extract", STEGO, C, MSG, C // 8, 100, None, 0, RES, 8)
     assert q[0][1] == 1
+
+
+CALLS = {
+    "one bit": (8192 * 64, 0, 0, 0, None),
+    "one bit, same misalignment": (8192 * 64, 3, 3, 0, None),
+    "one bit, other misalignment": (8192 * 64, 3, 0, 0, None),
+    "one bit, a few bytes": (40, 3, 0, 0, None),
+    "two bits": (8192 * 64, 0, 0, S.BITS(2), None),
+    "two bits, odd": (8192 * 64, 3, 5, S.BITS(2), None),
+    "one plane": (512 * 512 * 3, 0, 0, S.BITS(3) | S.PLANE_ONLY, (512, 512, 3, 1)),
+    "one plane of two": (512 * 512 * 2, 0, 0, S.PLANE_ONLY, (512, 512, 2, 1)),
+    "paper": (512 * 512 * 3, 0, 0, S.LAYOUT_PAPER2, (512, 512, 3, 1)),
+    "paper, two channels": (512 * 512 * 2, 0, 0, S.LAYOUT_PAPER2, (512, 512, 2, 1)),
+}
+
+
+@pytest.mark.parametrize("inplace", [False, True])
+@pytest.mark.parametrize("name", list(CALLS))
+def test_embed_behind_a_memset_is_no_dependent(L, name, inplace):
+    """Statistics without a slot (here: under capture) are zeroed by a memset right
+    before the kernel that adds to them, which is then an ordinary launch."""
+    C, at, out, flags, geom = CALLS[name]
+    out = at if inplace else out
+    g = S.Geom(*geom) if geom else None
+    geom = ctypes.addressof(g) if g else None
+    stego = COVER + out if inplace else STEGO + out
+    q = L.queued("stego_embed", COVER + at, stego, C, MSG, 4, geom, flags | S.FUSE_STATS, RES, 8,
+                 capturing=True)
+    at = [i for i, e in enumerate(q) if e[0] == "memset"]
+    assert len(at) == 1 and q[at[0]] == ("memset", 16)
+    assert at[0] == len(q) - 2 and q[-1][3] == 0, q
+    # with a slot: no memset, dependents only
+    q = L.queued("stego_embed", COVER + C, STEGO + C, C, MSG, 4, geom, flags | S.FUSE_STATS, RES, 8)
+    assert q and all(e[0] != "memset" and e[3] == 1 for e in q), q
+
+
+@pytest.mark.parametrize("n", [0, 100, 1 << 20])
+@pytest.mark.parametrize("at", [0, 5])
+def test_comparison_behind_a_memset_is_no_dependent(L, n, at):
+    q = L.queued("stego_changed_bytes", COVER + at, STEGO, n, RES, 8, capturing=True)
+    assert q[0] == ("memset", 16) and len(q) == 1 + (n > 0) and all(e[3] == 0 for e in q[1:])
+    if n:
+        q = L.queued("stego_changed_bytes", COVER + at, STEGO, n, RES, 8)
+        assert len(q) == 1 and q[0][3] == 1
