@@ -25,13 +25,13 @@ Shape g_shape[STEGO_OP_COUNT] = {
 };
 int g_sms[kMaxDevices];
 
-// Statistics slots: per device, the streams (by their process-unique
+// Statistics slots: per device and use, the streams (by their process-unique
 // stream ID, never reused, unlike a destroyed stream's handle) that own slots
-// 0..n-1, the device address of the slot array, and the context those
+// 0..n-1; per device, the address of the slot array and the context these
 // belong to.
-constexpr int kStatSlots = 256;
-unsigned long long g_slot_sid[kMaxDevices][kStatSlots];
-int g_slot_n[kMaxDevices];
+constexpr int kStatSlots = 256, kSlotUses = (int)SlotUse::kCount;
+unsigned long long g_slot_sid[kMaxDevices][kSlotUses][kStatSlots];
+int g_slot_n[kMaxDevices][kSlotUses];
 StatSlot *g_slot_base[kMaxDevices];
 unsigned long long g_slot_ctx[kMaxDevices];
 
@@ -244,11 +244,11 @@ cudaError_t write_result(stego_result *res, uint64_t msg_bytes, int status, cuda
 
 // Zero at load; each slot is cleared again by the last CTA of every launch
 // that used it.
-static __device__ stego::StatSlot g_stat_slots[stego::kStatSlots];
+static __device__ stego::StatSlot g_stat_slots[stego::kSlotUses * stego::kStatSlots];
 
 namespace stego {
 
-StatSlot *stats_slot(cudaStream_t s)
+StatSlot *stats_slot(cudaStream_t s, SlotUse use)
 {
     if (s == cudaStreamPerThread)
         return nullptr;
@@ -275,16 +275,19 @@ StatSlot *stats_slot(cudaStream_t s)
         if (cudaGetSymbolAddress(&p, g_stat_slots) != cudaSuccess || !p)
             return nullptr;
         g_slot_base[dev] = static_cast<StatSlot *>(p);
-        g_slot_n[dev] = 0;
+        std::memset(g_slot_n[dev], 0, sizeof(g_slot_n[dev]));
         g_slot_ctx[dev] = ctx;
     }
-    for (int i = 0; i < g_slot_n[dev]; ++i)
-        if (g_slot_sid[dev][i] == sid)
-            return g_slot_base[dev] + i;
-    if (g_slot_n[dev] == kStatSlots)
+    StatSlot *const base = g_slot_base[dev] + (int)use * kStatSlots;
+    unsigned long long *const sids = g_slot_sid[dev][(int)use];
+    int &n = g_slot_n[dev][(int)use];
+    for (int i = 0; i < n; ++i)
+        if (sids[i] == sid)
+            return base + i;
+    if (n == kStatSlots)
         return nullptr;
-    g_slot_sid[dev][g_slot_n[dev]] = sid;
-    return g_slot_base[dev] + g_slot_n[dev]++;
+    sids[n] = sid;
+    return base + n++;
 }
 
 } // namespace stego
@@ -392,7 +395,7 @@ int stego_embed(const uint8_t *d_cover, uint8_t *d_stego, uint64_t cover_bytes,
 
     cudaStream_t s = (cudaStream_t)stream;
     const Shape sh = shape_for(STEGO_OP_EMBED, nullptr);
-    StatSlot *slot = stats_slot(s); // statistics, tile counter
+    StatSlot *slot = stats ? stats_slot(s, SlotUse::kStats) : nullptr;
 
     if (layout == STEGO_LAYOUT_STREAM1 && (k != 1 || plane_only)) {
         if (cover_bytes == 0 || (!header && msg_bytes == 0 && inplace)) {
@@ -551,7 +554,7 @@ int stego_changed_bytes(const uint8_t *d_a, const uint8_t *d_b, uint64_t n, uint
     cudaStream_t s = (cudaStream_t)stream;
     if (n == 0)
         return cuda_status(cudaMemsetAsync(d_out2, 0, 2 * sizeof(uint64_t), s));
-    StatSlot *slot = stats_slot(s);
+    StatSlot *slot = stats_slot(s, SlotUse::kOther);
     const Shape sh = shape_for(STEGO_OP_CHANGED, nullptr);
     return cuda_status(changed_bytes(d_a, d_b, n, reinterpret_cast<unsigned long long *>(d_out2), sh, s, slot));
 }

@@ -115,25 +115,33 @@ struct StatSlot {
     unsigned long long pad;
 };
 
-// The slot of stream s on the current device, or nullptr: then the caller
-// zeroes res->changed/sse before the launch and the CTAs add into them.
+// What a slot is taken for.  The uses have slots of their own, so that streams
+// that only compare, or embed without statistics, leave the statistics theirs.
+enum class SlotUse {
+    kStats, // an embed's fused statistics (and its tile counter)
+    kOther, // a comparison's totals; the tile counter of an embed without statistics
+    kCount
+};
+
+// The slot of stream s on the current device, or nullptr: then totals are
+// zeroed before the launch and the CTAs add into them, and tiles are not claimed.
+// Taken only by calls that use it (it costs them some queries of the stream).
 // Slots are keyed by the stream's ID (cudaStreamGetId), which the runtime
 // never reuses, so a stream created after another was destroyed never
 // shares the old stream's slot (whose last launch may still be running).
 // nullptr for streams being captured into a graph (a replay may run beside
 // direct calls on the same stream), for the per-thread default stream
-// (one handle, several streams) and once every slot is taken (256 streams
-// per device; slots are never handed back, the later streams take the
+// (one handle, several streams) and once every slot of the use is taken (256
+// streams per device; slots are never handed back, the later streams take the
 // zeroing path).
-StatSlot *stats_slot(cudaStream_t s);
+StatSlot *stats_slot(cudaStream_t s, SlotUse use);
 
 // ---------------------------------------------------------------------------
 // Launchers (all stream-ordered, no synchronisation).  They return the CUDA
 // error of the launch.  `res` (nullable) receives msg_bytes = res_msg_bytes
 // and status STEGO_OK from block 0 of the launch; with `stats`, res->changed
 // and res->sse accumulate the changed-byte count and squared error (see
-// launch_counting).  `slot` is the stream's slot or nullptr, with or without
-// statistics (the tile counter is there too).
+// launch_counting).  `slot` is the stream's slot for statistics, or nullptr.
 // ---------------------------------------------------------------------------
 
 // STREAM1 embed.  n_bytes: bytes written (C out of place, T in place).
@@ -293,9 +301,13 @@ __device__ __forceinline__ void block_stats(unsigned long long a, unsigned long 
 // Whether tiles are claimed: with a slot, and more than four for each CTA (with
 // fewer the CTAs have no time to drift, and the barrier per tile costs more:
 // 25 MB at odd addresses 12.0 us, 13.3 claimed).
+__host__ __device__ __forceinline__ bool enough_tiles(uint64_t ntiles, uint32_t ctas)
+{
+    return ntiles > 4ull * ctas;
+}
 __device__ __forceinline__ bool tiles_claimed(const StatSlot *slot, uint32_t ntiles)
 {
-    return slot && ntiles > 4u * gridDim.x;
+    return slot && enough_tiles(ntiles, gridDim.x);
 }
 
 // Calls body(tile) for this CTA's tiles of ntiles, all its threads together:

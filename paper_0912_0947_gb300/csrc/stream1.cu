@@ -309,6 +309,16 @@ constexpr int kShiftThreads = 256;
 
 } // namespace
 
+// An embed kernel over ntiles tiles.  Without statistics the stream's slot is taken
+// only for the tile counter, where there are enough tiles to claim.
+static cudaError_t launch_tiles(const void *k, int grid, int threads, void **args, EmbedArgs &e,
+                                bool stats, uint64_t ntiles, cudaStream_t s)
+{
+    if (!stats)
+        e.slot = enough_tiles(ntiles, (uint32_t)grid) ? stats_slot(s, SlotUse::kOther) : nullptr;
+    return launch_counting(k, dim3(grid), dim3(threads), args, 0, s, stats ? e.res : nullptr, e.slot);
+}
+
 cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uint64_t t_bytes,
                      const uint8_t *msg, uint64_t slen, bool header, uint32_t nbits, bool stats,
                      stego_result *res, uint64_t res_msg_bytes, const Shape &sh, cudaStream_t s,
@@ -344,7 +354,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvec = n_bytes >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvec > 0 ? nvec : 1,
                                          (uint64_t)T * vec);
-        return launch_counting(k, dim3(grid), dim3(T), args, 0, s, stats ? res : nullptr, slot);
+        return launch_tiles(k, grid, T, args, e, stats, (nvec + T * vec - 1) / (T * vec), s);
     }
     // heads up to a 128-byte boundary of the stego, so that a warp's vectors are
     // whole cache lines (16-byte boundaries in a small cover)
@@ -357,7 +367,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvb = (n_bytes - h) >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvb, (uint64_t)T * kShiftV);
         void *sargs[] = {&e, (void *)&h};
-        return launch_counting(k, dim3(grid), dim3(T), sargs, 0, s, stats ? res : nullptr, slot);
+        return launch_tiles(k, grid, T, sargs, e, stats, (nvb + T * kShiftV - 1) / (T * kShiftV), s);
     }
     const uint32_t hs = (uint32_t)(-(uintptr_t)stego & line);
     if (cover != stego && n_bytes >= (uint64_t)hs + 16u) {
@@ -374,7 +384,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         const uint64_t nvb = (n_bytes - hs) >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvb, (uint64_t)T * F);
         void *fargs[] = {&e, (void *)&hs, (void *)&sel};
-        return launch_counting(k, dim3(grid), dim3(T), fargs, 0, s, stats ? res : nullptr, slot);
+        return launch_tiles(k, grid, T, fargs, e, stats, (nvb + T * F - 1) / (T * F), s);
     }
     const void *k = stats ? (const void *)embed_bytes<true> : (const void *)embed_bytes<false>;
     const uint64_t units = (n_bytes + 7) >> 3;

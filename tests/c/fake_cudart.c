@@ -13,7 +13,7 @@
 
 static char g_log[1 << 16];
 static size_t g_len;
-static int g_capturing;
+static int g_capturing, g_id_queries;
 static char g_symbols[1 << 20] __attribute__((aligned(256)));
 static struct { const void *host; const char *name; } g_kernel[512];
 static int g_kernels;
@@ -28,7 +28,8 @@ static void put(const char *line)
 }
 
 const char *fake_log(void) { return g_log; }
-void fake_reset(int capturing) { g_len = 0; g_log[0] = 0; g_capturing = capturing; }
+void fake_reset(int capturing) { g_len = 0; g_log[0] = 0; g_capturing = capturing; g_id_queries = 0; }
+int fake_id_queries(void) { return g_id_queries; }
 int fake_wave(void) { return SMS * PER_SM; }
 
 static const char *kernel_name(const void *f)
@@ -119,7 +120,12 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, enum cudaStreamCaptureStatus *
     *st = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
-cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long *id) { *id = (uintptr_t)s; return cudaSuccess; }
+cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long *id)
+{
+    ++g_id_queries;
+    *id = (uintptr_t)s;
+    return cudaSuccess;
+}
 cudaError_t cudaGetSymbolAddress(void **p, const void *s) { (void)s; *p = g_symbols; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void *f, enum cudaFuncAttribute a, int v) { (void)f; (void)a; (void)v; return cudaSuccess; }

@@ -79,3 +79,26 @@ def test_comparison_behind_a_memset_is_no_dependent(L, n, at):
     if n:
         q = L.queued("stego_changed_bytes", COVER + at, STEGO, n, RES, 8)
         assert len(q) == 1 and q[0][3] == 1
+
+
+def test_slots_are_the_statistics():
+    """Embeds without statistics and comparisons on hundreds of streams leave every
+    slot to embeds with statistics; those that use no slot do not ask for one."""
+    L = Launches()  # slots are never handed back: a library of its own
+    geom = S.Geom(512, 512, 3, 1)
+    g = ctypes.addressof(geom)
+    for s in range(1, 301):
+        L.queued("stego_embed", COVER, STEGO, 1 << 30, MSG, 4, None, 0, None, s << 8)
+        L.queued("stego_embed", COVER, STEGO, 512 * 512 * 3, MSG, 4, g, S.LAYOUT_PAPER2, None, s << 8)
+        L.queued("stego_changed_bytes", COVER, STEGO, 1 << 20, RES, s << 8)
+    for s in range(1001, 1257):
+        q = L.queued("stego_embed", COVER, STEGO, 1 << 20, MSG, 4, None, S.FUSE_STATS, RES, s << 8)
+        assert len(q) == 1, (s, q)
+    q = L.queued("stego_embed", COVER, STEGO, 1 << 20, MSG, 4, None, S.FUSE_STATS, RES, 2000 << 8)
+    assert q[0] == ("memset", 16)  # the 257th
+    for C, flags, gm, asks in ((1 << 30, 0, None, 1), (1 << 20, 0, None, 0),
+                               (1 << 30, S.BITS(2), None, 0),
+                               (512 * 512 * 3, S.LAYOUT_PAPER2, g, 0),
+                               (512 * 512 * 3, S.PLANE_ONLY, g, 0)):
+        L.queued("stego_embed", COVER, STEGO, C, MSG, 4, gm, flags, None, 3000 << 8)
+        assert L.lib.fake_id_queries() == asks, (C, flags)
