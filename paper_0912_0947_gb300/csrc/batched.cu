@@ -85,8 +85,11 @@ __device__ __forceinline__ uint64_t whole_rounds(uint64_t per)
 // Most tiles per claim, of the stream layout and of the paper's (see
 // claim_size): long runs while there are many tiles, so that a large batch pays
 // few set-ups, and single tiles where there are few, so that a small batch
-// spreads over as many CTAs as there are and all end together.
-constexpr uint32_t kChunk = 2u, kPaperChunk = 4u;
+// spreads over as many CTAs as there are and all end together.  kLargeChunk: of
+// embeds in shapes other than the default one, whose few CTAs per SM leave the time
+// between two claims in the open (1024 uneven covers, 512 threads, statistics, four
+// and two vectors: 826 and 734 us with two tiles, 798 and 721 with four).
+constexpr uint32_t kChunk = 2u, kPaperChunk = 4u, kLargeChunk = 4u;
 
 // Workspace: head (64 B), aligned-stream, paper and misaligned-stream tile
 // offsets (n+1 each), per-descriptor info (64 B each, 16-byte aligned).
@@ -541,13 +544,6 @@ __device__ __forceinline__ void flush_stats(unsigned long long &changed, unsigne
     sse = 0;
 }
 
-// The claim loop shared by both directions: calls body(d, first, count) for
-// the tiles of the chunks this CTA claims, in order.  MERGE: once for every run
-// of `count` consecutive tiles of one descriptor, one set-up for all of them (a
-// call per tile cost the paper layout's kernels as many instructions as a
-// round of their threads); else tile by tile, count = 1 (the stream kernels'
-// set-up is a few loads, and merged ranges cost persist_embed<4, true> two
-// registers and with them the third CTA per SM).
 // Tiles of a claim: a quarter of the CTA's share of `left` tiles, at most MAX.
 template <uint32_t MAX>
 __device__ __forceinline__ uint32_t claim_size(unsigned long long left)
@@ -570,14 +566,19 @@ __device__ __forceinline__ uint32_t split_shift(unsigned long long total, uint32
     return s;
 }
 
-// (`total` tiles, each in 2^shift parts; `first` counts parts of the
-// descriptor's tiles; parts are claimed and taken singly.)
-template <bool MERGE, typename Body>
+// The claim loop shared by both directions, over `total` tiles, each in 2^shift
+// parts: calls body for the parts of the chunks this CTA claims, in order.  MERGE:
+// body(d, first, count) once for every run of `count` consecutive tiles of one
+// descriptor, one set-up for all of them (a call per tile cost the paper layout's
+// kernels as many instructions as a round of their threads); parts of a tile, and
+// the stream kernels' tiles, singly: body(d, first) (their set-up is a few loads,
+// and merged ranges cost persist_embed<4, true> two registers and with them the
+// third CTA per SM).  `first` counts the descriptor's parts.
+template <bool MERGE, uint32_t MAX, typename Body>
 __device__ __forceinline__ void claim_loop(const unsigned long long *start,
                                            unsigned long long total, uint32_t shift,
                                            unsigned long long *counter, uint32_t n, Body &&body)
 {
-    constexpr uint32_t MAX = MERGE ? kPaperChunk : kChunk;
     __shared__ unsigned long long s_claim;
     __shared__ uint32_t s_count;
     const unsigned long long parts = total << shift;
@@ -608,11 +609,16 @@ __device__ __forceinline__ void claim_loop(const unsigned long long *start,
             while (start[d + 1] <= t >> shift)
                 ++d;
             const unsigned long long first = t - (start[d] << shift);
-            uint32_t cnt = 1;
-            if (MERGE && shift == 0)
-                cnt = (uint32_t)((start[d + 1] < c1 ? start[d + 1] : c1) - t);
-            t += cnt;
-            body(d, first, cnt);
+            if constexpr (MERGE) {
+                uint32_t cnt = 1;
+                if (shift == 0)
+                    cnt = (uint32_t)((start[d + 1] < c1 ? start[d + 1] : c1) - t);
+                t += cnt;
+                body(d, first, cnt);
+            } else {
+                ++t;
+                body(d, first);
+            }
         }
         __syncthreads(); // the next claim is visible
     }
@@ -737,9 +743,12 @@ __device__ __forceinline__ void paper_extract_tile(const stego_desc &D, const De
 }
 
 // Four vectors per thread in CTAs of at most 256 threads (the default shape)
-// keep 80 registers, three CTAs per SM: 82 cost 13% of the uneven batch.
+// keep 80 registers, three CTAs per SM: 82 cost 13% of the uneven batch.  No bound
+// for the others: with one CTA per SM as theirs the compiler took 56-91 registers
+// in place of 32-82 (1024 uneven covers, 512 threads, no statistics, four vectors
+// 794 us, so 654; with statistics, two vectors 1011, so 721).
 template <int V, bool STATS, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 1) persist_embed(const stego_desc *descs, uint32_t n,
+__global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 0) persist_embed(const stego_desc *descs, uint32_t n,
                                                      stego_result *results, WsView ws,
                                                      uint32_t tile_bytes)
 {
@@ -749,8 +758,8 @@ __global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 1) persist_embe
     uint32_t stat_d = 0xFFFFFFFFu;
     const unsigned long long total = ws.head->total;
     const uint32_t shift = split_shift(total, tile_bytes), part_bytes = tile_bytes >> shift;
-    claim_loop<false>(ws.start, total, shift, &ws.head->counter, n,
-               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
+    claim_loop<false, SMALL ? kChunk : kLargeChunk>(ws.start, total, shift, &ws.head->counter, n,
+               [&](uint32_t d, unsigned long long lt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
             stat_d = d;
@@ -768,7 +777,7 @@ __global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 1) persist_embe
         a.nbits = inf.nbits;
         a.msg_even = (inf.bits & kMsgEven) ? 1u : 0u;
         a.pad = 0;
-        const uint64_t b0 = lt * part_bytes, be = b0 + (uint64_t)cnt * part_bytes;
+        const uint64_t b0 = lt * part_bytes, be = b0 + part_bytes;
         const uint64_t b1 = be < inf.n_bytes ? be : inf.n_bytes;
         if (b0 >= b1)
             return; // a part past the cover's end
@@ -794,8 +803,8 @@ __global__ void __launch_bounds__(512) persist_extract(const stego_desc *descs, 
     allow_dependents();
     const unsigned long long total = ws.head->total;
     const uint32_t shift = split_shift(total, tile_bytes), part_bytes = tile_bytes >> shift;
-    claim_loop<false>(ws.start, total, shift, &ws.head->counter, n,
-               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
+    claim_loop<false, kChunk>(ws.start, total, shift, &ws.head->counter, n,
+               [&](uint32_t d, unsigned long long lt) {
         const stego_desc &D = descs[d];
         const DescInfo inf = ws.info[d];
         s1::ExtractView x;
@@ -805,7 +814,7 @@ __global__ void __launch_bounds__(512) persist_extract(const stego_desc *descs, 
         x.base = (inf.bits & kHeader) ? 32u : 0u;
         x.msg_even = (inf.bits & kMsgEven) ? 1u : 0u;
         x.pad = 0;
-        const uint64_t b0 = lt * part_bytes, be = b0 + (uint64_t)cnt * part_bytes;
+        const uint64_t b0 = lt * part_bytes, be = b0 + part_bytes;
         const uint64_t b1 = be < inf.n_bytes ? be : inf.n_bytes;
         if (b0 >= b1)
             return; // a part past the cover's end
@@ -841,11 +850,11 @@ __device__ __forceinline__ void mis_funnel(const s1::EmbedView &a, uint32_t h, u
                                                  blockDim.x >> 5, changed, sse);
 }
 
-// Tiles lt .. lt + cnt - 1 of a misaligned stream cover (the CTA's threads together).
+// Part lt of a misaligned stream cover (the CTA's threads together).
 template <bool STATS>
 __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescInfo &inf,
-                                               unsigned long long lt, uint32_t cnt,
-                                               uint32_t shift, unsigned long long &changed,
+                                               unsigned long long lt, uint32_t shift,
+                                               unsigned long long &changed,
                                                unsigned long long &sse)
 {
         s1::EmbedView a;
@@ -863,7 +872,7 @@ __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescIn
         const uint64_t nvb = (inf.n_bytes - h) >> 4;
         // (a misaligned tile is tile_bytes / 16 vectors: whole parts, see split_shift)
         const uint64_t per = inf.per_tile >> shift;
-        const uint64_t j0 = lt * per, je = j0 + (uint64_t)cnt * per;
+        const uint64_t j0 = lt * per, je = j0 + per;
         const uint64_t j1 = je < nvb ? je : nvb;
         if (j0 >= j1)
             return; // a part past the cover's end
@@ -893,8 +902,7 @@ __device__ __forceinline__ void mis_embed_tile(const stego_desc &D, const DescIn
 }
 
 __device__ __forceinline__ void mis_extract_tile(const stego_desc &D, const DescInfo &inf,
-                                                 unsigned long long lt, uint32_t cnt,
-                                                 uint32_t shift)
+                                                 unsigned long long lt, uint32_t shift)
 {
         s1::ExtractView x;
         x.st = D.cover;
@@ -905,7 +913,7 @@ __device__ __forceinline__ void mis_extract_tile(const stego_desc &D, const Desc
         x.pad = 0;
         const uint64_t np = inf.len >> 1;
         const uint64_t per = inf.per_tile >> shift;
-        const uint64_t p0 = lt * per, pe = p0 + (uint64_t)cnt * per;
+        const uint64_t p0 = lt * per, pe = p0 + per;
         const uint64_t p1 = pe < np ? pe : np;
         if (p0 >= p1)
             return; // a part past the message's end
@@ -941,13 +949,13 @@ __global__ void __launch_bounds__(kMisEmbedThreads, kMisEmbedMinCtas)
     uint32_t stat_d = 0xFFFFFFFFu;
     const unsigned long long total = ws.head->total_m;
     const uint32_t shift = split_shift(total, tile_bytes);
-    claim_loop<false>(ws.start_m, total, shift, &ws.head->counter_m, n,
-               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
+    claim_loop<false, kChunk>(ws.start_m, total, shift, &ws.head->counter_m, n,
+               [&](uint32_t d, unsigned long long lt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
             stat_d = d;
         }
-        mis_embed_tile<STATS>(descs[d], ws.info[d], lt, cnt, shift, changed, sse);
+        mis_embed_tile<STATS>(descs[d], ws.info[d], lt, shift, changed, sse);
     });
     if (STATS)
         flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
@@ -961,9 +969,9 @@ __global__ void __launch_bounds__(kMisExtractThreads)
     allow_dependents();
     const unsigned long long total = ws.head->total_m;
     const uint32_t shift = split_shift(total, tile_bytes);
-    claim_loop<false>(ws.start_m, total, shift, &ws.head->counter_m, n,
-               [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
-        mis_extract_tile(descs[d], ws.info[d], lt, cnt, shift);
+    claim_loop<false, kChunk>(ws.start_m, total, shift, &ws.head->counter_m, n,
+               [&](uint32_t d, unsigned long long lt) {
+        mis_extract_tile(descs[d], ws.info[d], lt, shift);
     });
 }
 
@@ -988,7 +996,7 @@ __global__ void __launch_bounds__(kP2Threads, 4) persist_p2_embed(const stego_de
     uint32_t stat_d = 0xFFFFFFFFu;
     const unsigned long long total = ws.head->total_p;
     const uint32_t shift = split_shift(total, tile_bytes);
-    claim_loop<true>(ws.start_p, total, shift, &ws.head->counter_p, n,
+    claim_loop<true, kPaperChunk>(ws.start_p, total, shift, &ws.head->counter_p, n,
                [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         if (STATS && d != stat_d) {
             flush_stats(changed, sse, stat_d < n ? results + stat_d : nullptr);
@@ -1007,7 +1015,7 @@ __global__ void __launch_bounds__(kP2Threads, 4) persist_p2_extract(const stego_
     allow_dependents();
     const unsigned long long total = ws.head->total_p;
     const uint32_t shift = split_shift(total, tile_bytes);
-    claim_loop<true>(ws.start_p, total, shift, &ws.head->counter_p, n,
+    claim_loop<true, kPaperChunk>(ws.start_p, total, shift, &ws.head->counter_p, n,
                [&](uint32_t d, unsigned long long lt, uint32_t cnt) {
         paper_extract_tile(descs[d], ws.info[d], lt, cnt, shift);
     });
