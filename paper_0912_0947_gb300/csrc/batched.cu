@@ -71,9 +71,10 @@ constexpr uint32_t kHeader = 1u, kVec = 2u, kMsgEven = 4u;
 // (stego vectors joined from cover vector pairs); otherwise the same
 // misalignment (vectors after a scalar head)
 constexpr uint32_t kFunnel = 8u;
-// paper-layout work kinds (0 = the one-bit stream layout)
+// paper-layout work kinds (0 = the one-bit stream layout); kP2RunsAligned: see
+// p2::runs_aligned
 constexpr uint32_t kP2Units = 1u, kP2RowsCopy = 2u, kP2Rows = 3u, kP2Runs = 4u, kP2RowsX = 5u,
-                   kP2UnitsInPlace = 6u;
+                   kP2UnitsInPlace = 6u, kP2RunsAligned = 7u;
 // Threads of the paper-layout persistent kernels' CTAs.  Unit and run tiles
 // hold a whole number of CTA rounds (tile_bytes rounded down), so that no
 // round runs with idle threads in the middle of a cover.
@@ -362,7 +363,7 @@ __device__ __forceinline__ Tiles prep_extract(const stego_desc &D, uint32_t d, s
             const uint64_t per = whole_rounds(tile_bytes / (64u * D.geom.channels)
                                                   ? tile_bytes / (64u * D.geom.channels)
                                                   : 1u);
-            inf.mode = kP2Runs;
+            inf.mode = p2::runs_aligned(v) ? kP2RunsAligned : kP2Runs;
             inf.per_tile = (uint32_t)per;
             tiles = (runs + per - 1) / per;
         } else {
@@ -701,9 +702,9 @@ __device__ __forceinline__ void paper_embed_tile(const stego_desc &D, const Desc
         // and ran slower (600 video frames: 1.53 against 1.26 ms), and so did
         // the cp.async pipeline of the single-cover kernel (1.34-1.83 ms)
         switch (inf.channels) {
-        case 1: p2::units_embed<1, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
-        case 3: p2::units_embed<3, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
-        default: p2::units_embed<4, STATS, 1, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
+        case 1: p2::units_embed<1, STATS, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
+        case 3: p2::units_embed<3, STATS, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
+        default: p2::units_embed<4, STATS, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
         }
         if (b0 == 0 || b1 >= inf.n_bytes)
             p2::edge_bytes<STATS>(job.v, job.f, b0 == 0, b1 >= inf.n_bytes, changed, sse);
@@ -726,16 +727,37 @@ __device__ __forceinline__ void paper_extract_tile(const stego_desc &D, const De
                                                    unsigned long long lt, uint32_t cnt,
                                                  uint32_t shift)
 {
-    const PaperJob &job = paper_job(D, inf, false);
     uint64_t b0, b1;
     paper_part(inf, lt, cnt, shift, b0, b1);
-    if (inf.mode == kP2Runs) {
+    if (inf.mode == kP2RunsAligned) {
+        // the full rows need so little of the cover that each thread reads it for
+        // itself: without the barriers around paper_job, 300 HD frames 188 -> 176 us
+        p2::View v;
+        v.src = D.cover;
+        v.msg_out = D.msg;
+        v.W = inf.W;
+        v.Q = inf.W / 4u;
+        v.plane = inf.plane;
+        v.R = (uint32_t)inf.t_bytes;
+        v.L_last = (uint32_t)(inf.t_bytes >> 32);
+        const uint64_t full = p2::aligned_full_runs(v), ke = b1 < full ? b1 : full;
+        switch (inf.channels) {
+        case 1: p2::aligned_runs<1, 4, true>(v, b0 + threadIdx.x, ke, blockDim.x); break;
+        case 3: p2::aligned_runs<3, kBatchAligned, true>(v, b0 + threadIdx.x, ke, blockDim.x); break;
+        default: p2::aligned_runs<4, kBatchAligned, true>(v, b0 + threadIdx.x, ke, blockDim.x); break;
+        }
+        if (b1 <= full || v.L_last == v.Q)
+            return;
+        b0 = b0 > full ? b0 : full; // the last row's
+    }
+    const PaperJob &job = paper_job(D, inf, false);
+    if (inf.mode == kP2Runs || inf.mode == kP2RunsAligned) {
         const uint64_t runs = p2::run_count(job.v);
         const uint64_t k0 = b0 + threadIdx.x, k1 = b1 < runs ? b1 : runs;
         switch (inf.channels) {
-        case 1: p2::runs_extract<1, 4, 1>(job.v, k0, k1, blockDim.x); break;
-        case 3: p2::runs_extract<3, kBatchAligned, kBatchQuarters>(job.v, k0, k1, blockDim.x); break;
-        default: p2::runs_extract<4, kBatchAligned, kBatchQuarters>(job.v, k0, k1, blockDim.x); break;
+        case 1: p2::other_runs<1, 1, true>(job.v, k0, k1, blockDim.x); break;
+        case 3: p2::other_runs<3, kBatchQuarters, true>(job.v, k0, k1, blockDim.x); break;
+        default: p2::other_runs<4, kBatchQuarters, true>(job.v, k0, k1, blockDim.x); break;
         }
     } else {
         p2::rows_extract(job.v, (uint32_t)b0, (uint32_t)(b1 < job.v.R ? b1 : job.v.R), 1);
@@ -979,11 +1001,12 @@ __global__ void __launch_bounds__(kMisExtractThreads)
 // the stream kernels): tiles of units, rows or runs, claimed like above.
 // Capped at 64 registers for four CTAs per SM (1024 covers of sides 64 to 4096,
 // half RGB: embed 960 us against 1023 with three CTAs at 80 registers, 1107
-// with two, although it spills; extract 381 against 410).  One unit or run at a
+// with two, although it spills; extract of 300 frames 854 wide 105 against 114, of
+// the covers 379 against 364).  One unit or run at a
 // time: with four CTAs the warps hide the latency, and two in flight were
 // slower.  With rows that are not whole vectors copied and then scattered byte
-// by byte the same batch took 2823 us (embed) and 505 us (extract), now 896
-// and 388; large RGB covers run at 0.75 of the copy rate, gray ones, with
+// by byte the same batch took 2823 us (embed) and 505 us (extract), now 893
+// and 371; large RGB covers run at 0.75 of the copy rate, gray ones, with
 // three times the units per byte, at 0.53.
 template <bool STATS>
 __global__ void __launch_bounds__(kP2Threads, 4) persist_p2_embed(const stego_desc *descs, uint32_t n,

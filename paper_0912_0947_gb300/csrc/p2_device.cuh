@@ -328,18 +328,21 @@ __host__ __device__ constexpr uint32_t stage_vectors()
     return kStageWarps * 2 * (unit_stage_slots<CH>() + 1);
 }
 
-// One pass over units k = k_first + i*step (+ u*blockDim.x, u < UT), k <
-// k_end, each thread on its own units: every load of an iteration (cover,
-// then message) is issued before any arithmetic.  With one channel the lanes'
-// single-vector units are consecutive (coalesced); with three or four a lane's
-// unit lies 16*CH bytes from its neighbour's, which units_embed_async avoids
-// and the batched kernels accept for their register budget.  Cover and stego
-// at different addresses mod 16: the vector after the unit's own is loaded too
-// (the neighbour's first: an L1 hit) and the bytes joined.  Out of place every
-// unit is written (units without carrying pixels are copied); in place
-// (INPLACE) k_end is cut to the carrying units, each unit read and written
-// back by the same thread.
-template <int CH, bool STATS, int UT, bool INPLACE = false, bool LEAD = false>
+// One pass over units k = k_first + i*step < k_end, each thread on its own units:
+// every load of a unit (cover, then message) is issued before any arithmetic.  With
+// one channel the lanes' single-vector units are consecutive (coalesced); with
+// three or four a lane's unit lies 16*CH bytes from its neighbour's, which
+// units_embed_async avoids and the batched kernels accept for their register
+// budget.  Cover and stego at different addresses mod 16: the vector after the
+// unit's own is loaded too (the neighbour's first: an L1 hit) and the bytes joined.
+// Out of place every unit is written (units without carrying pixels are copied); in
+// place (INPLACE) k_end is cut to the carrying units, each unit read and written
+// back by the same thread.  BATCHED: three channels' plane byte at unit byte 0 (see
+// plan_units' lead), and a unit's row by a division each: kept from unit to unit by
+// additions it costs registers that the batched kernels spill (300 HD frames 645 us,
+// so 626; one channel in the single-cover kernel, which does not spill, 31.0
+// and 32.1).
+template <int CH, bool STATS, bool INPLACE = false, bool BATCHED = false>
 __device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32_t k_first,
                                             uint32_t k_end, uint32_t step,
                                             unsigned long long &changed, unsigned long long &sse)
@@ -349,57 +352,41 @@ __device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32
         k_end = carry;
     if (k_first >= k_end)
         return;
-    const PlaneSel sel = LEAD && CH == 3 ? make_sel(3, 0) : f.sel;
+    const PlaneSel sel = BATCHED && CH == 3 ? make_sel(3, 0) : f.sel;
     const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src + f.h - f.d);
     uint4 *dst = reinterpret_cast<uint4 *>(a.dst + f.h);
-    // row and column of the thread's first pixel, kept by additions
-    const uint64_t x = f.x0 + 16ull * k_first;
-    uint32_t r0 = row_of(x, a.W), c0 = (uint32_t)(x - (uint64_t)r0 * a.W);
-    const uint32_t tr = UT > 1 ? 16u * blockDim.x / a.W : 0u;
-    const uint32_t tc = UT > 1 ? 16u * blockDim.x - tr * a.W : 0u;
+    // row and column of the unit's first pixel
+    const uint64_t x0 = f.x0 + 16ull * k_first;
+    uint32_t r = row_of(x0, a.W), col = (uint32_t)(x0 - (uint64_t)r * a.W);
     const uint32_t sr = 16u * step / a.W, sc = 16u * step - sr * a.W; // 16 * step < 2^32
-    for (uint32_t k0 = k_first; k0 < k_end; k0 += step) {
-        uint32_t c[UT][4 * CH + 4];
+    for (uint32_t k = k_first; k < k_end; k += step) {
+        uint32_t c[4 * CH + 4], o[4 * CH];
 #pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint32_t k = k0 + u * blockDim.x;
-            if (k < k_end) {
-#pragma unroll
-                for (int q = 0; q < CH; ++q)
-                    set_vec(c[u], q, __ldcs(src + (uint64_t)k * CH + q));
-                if (!INPLACE && f.d)
-                    set_vec(c[u], CH, __ldcs(src + (uint64_t)k * CH + CH));
-            }
+        for (int q = 0; q < CH; ++q)
+            set_vec(c, q, __ldcs(src + (uint64_t)k * CH + q));
+        if (!INPLACE && f.d)
+            set_vec(c, CH, __ldcs(src + (uint64_t)k * CH + CH));
+        if constexpr (BATCHED) {
+            const uint64_t x = f.x0 + 16ull * k;
+            r = row_of(x, a.W);
+            col = (uint32_t)(x - (uint64_t)r * a.W);
         }
-        UnitJob J[UT];
-        uint32_t r = r0, col = c0;
+        UnitJob J;
+        plan_unit(a, k < carry, r, col, J);
+        if (!INPLACE && f.d) {
+            join_unit<CH>(c, f.d, o);
+        } else {
 #pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint32_t k = k0 + u * blockDim.x;
-            if (u > 0)
-                rc_add(r, col, tr, tc, a.W);
-            plan_unit(a, k < k_end && k < carry, r, col, J[u]);
+            for (int q = 0; q < 4 * CH; ++q)
+                o[q] = c[q];
         }
+        if (J.mode)
+            embed_unit<CH, STATS>(a, J, sel, o, changed, sse);
 #pragma unroll
-        for (int u = 0; u < UT; ++u) {
-            const uint32_t k = k0 + u * blockDim.x;
-            if (k >= k_end)
-                continue;
-            uint32_t o[4 * CH];
-            if (!INPLACE && f.d) {
-                join_unit<CH>(c[u], f.d, o);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4 * CH; ++q)
-                    o[q] = c[u][q];
-            }
-            if (J[u].mode)
-                embed_unit<CH, STATS>(a, J[u], sel, o, changed, sse);
-#pragma unroll
-            for (int q = 0; q < CH; ++q)
-                __stcs(dst + (uint64_t)k * CH + q, get_vec(o, q));
-        }
-        rc_add(r0, c0, sr, sc, a.W);
+        for (int q = 0; q < CH; ++q)
+            __stcs(dst + (uint64_t)k * CH + q, get_vec(o, q));
+        if constexpr (!BATCHED)
+            rc_add(r, col, sr, sc, a.W);
     }
 }
 
@@ -691,19 +678,25 @@ __device__ __forceinline__ void get_pairs(const uint32_t (&w)[4 * CH], uint32_t 
 }
 
 // Runs k = k_first + i*step < k_end of an aligned layout's full rows, GA
-// quarters' vectors at a time.
-template <int CH, int PLANE, int GA>
+// quarters' vectors at a time.  BATCHED: a run's row and block by a 32-bit division,
+// else kept by additions (8192x8192x3 33.1 us, 33.4 by divisions; in the batched
+// kernel the additions cost registers that it spills: 1024 paper covers 380 us, by
+// divisions here and in other_runs 372).
+template <int CH, int PLANE, int GA, bool BATCHED>
 __device__ __forceinline__ void full_runs(const View &a, uint64_t k_first, uint64_t k_end,
                                           uint32_t step)
 {
     const uint32_t rpr = a.Q / 16u, W16 = a.W / 16u;
     const uint32_t stride = rpr * CH; // vectors from quarter to quarter
-    // row and block of the run, kept by additions
     uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
     const uint32_t dr = step / rpr, db = step - dr * rpr;
     const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src);
     uint4 *out = reinterpret_cast<uint4 *>(a.msg_out);
     for (uint64_t k = k_first; k < k_end; k += step) {
+        if constexpr (BATCHED) {
+            r = row_of(k, rpr);
+            b = (uint32_t)(k - (uint64_t)r * rpr);
+        }
         const uint4 *A = src + ((uint64_t)r * W16 + b) * CH;
         uint32_t M[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
@@ -730,42 +723,26 @@ __device__ __forceinline__ void full_runs(const View &a, uint64_t k_first, uint6
             }
         }
         out[k] = make_uint4(M[0], M[1], M[2], M[3]);
-        rc_add(r, b, dr, db, rpr);
+        if constexpr (!BATCHED)
+            rc_add(r, b, dr, db, rpr);
     }
 }
 
-// Extraction over runs k = k_first + i*step < k_end: those of an aligned
-// layout's full rows GA quarters' vectors at a time, then all others G (each
-// part with an index of its own: one carried from the first to the second cost
-// the first its registers, 300 video frames 199 against 180 us).
-template <int CH, int GA, int G>
-__device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, uint64_t k_end,
-                                             uint32_t step)
+// Runs k = k_first + i*step < k_end of any layout, G quarters' vectors at a time
+// (BATCHED: see full_runs).
+template <int CH, int G, bool BATCHED>
+__device__ __forceinline__ void other_runs(const View &a, uint64_t k_first, uint64_t k_end,
+                                           uint32_t step)
 {
-    if (k_first >= k_end)
-        return;
-    if (runs_aligned(a)) {
-        const uint64_t full = (uint64_t)(a.L_last == a.Q ? a.R : a.R - 1) * (a.Q / 16u);
-        const uint64_t ke = k_end < full ? k_end : full;
-        switch (CH == 1 ? 0u : a.plane) {
-        case 0: full_runs<CH, 0, GA>(a, k_first, ke, step); break;
-        case 1: full_runs<CH, CH == 1 ? 0 : 1, GA>(a, k_first, ke, step); break;
-        case 2: full_runs<CH, CH == 1 ? 0 : 2, GA>(a, k_first, ke, step); break;
-        default: full_runs<CH, CH == 4 ? 3 : 0, GA>(a, k_first, ke, step); break;
-        }
-        if (k_end <= full)
-            return;
-        if (k_first < full) // the first run past the full rows
-            k_first += (full - k_first + step - 1) / step * step;
-        if (k_first >= k_end)
-            return;
-    }
-    // row and block of the run, kept by additions
     const uint32_t rpr = run_row(a);
     uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
     const uint32_t dr = step / rpr, db = step - dr * rpr;
     const uint64_t C = (uint64_t)a.W * a.H * CH;
     for (uint64_t k = k_first; k < k_end; k += step) {
+        if constexpr (BATCHED) {
+            r = row_of(k, rpr);
+            b = (uint32_t)(k - (uint64_t)r * rpr);
+        }
         const uint32_t L = row_len(a, r);
         uint8_t *mrow = a.msg_out + (uint64_t)r * a.Q;
         const int64_t j0 = 16ll * b - (int64_t)((uintptr_t)mrow & 15u); // row byte of the block's first
@@ -794,8 +771,48 @@ __device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, ui
                 }
             }
         }
-        rc_add(r, b, dr, db, rpr);
+        if constexpr (!BATCHED)
+            rc_add(r, b, dr, db, rpr);
     }
+}
+
+// Runs of an aligned layout's full rows.
+__host__ __device__ inline uint64_t aligned_full_runs(const View &a)
+{
+    return (uint64_t)(a.L_last == a.Q ? a.R : a.R - 1) * (a.Q / 16u);
+}
+
+// Runs k = k_first + i*step < k_end of an aligned layout's full rows, GA quarters'
+// vectors at a time.
+template <int CH, int GA, bool BATCHED>
+__device__ __forceinline__ void aligned_runs(const View &a, uint64_t k_first, uint64_t k_end,
+                                             uint32_t step)
+{
+    switch (CH == 1 ? 0u : a.plane) {
+    case 0: full_runs<CH, 0, GA, BATCHED>(a, k_first, k_end, step); break;
+    case 1: full_runs<CH, CH == 1 ? 0 : 1, GA, BATCHED>(a, k_first, k_end, step); break;
+    case 2: full_runs<CH, CH == 1 ? 0 : 2, GA, BATCHED>(a, k_first, k_end, step); break;
+    default: full_runs<CH, CH == 4 ? 3 : 0, GA, BATCHED>(a, k_first, k_end, step); break;
+    }
+}
+
+// Extraction over runs k = k_first + i*step < k_end: those of an aligned layout's
+// full rows GA quarters' vectors at a time, then all others G.
+template <int CH, int GA, int G>
+__device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, uint64_t k_end,
+                                             uint32_t step)
+{
+    if (k_first >= k_end)
+        return;
+    if (runs_aligned(a)) {
+        const uint64_t full = aligned_full_runs(a);
+        aligned_runs<CH, GA, false>(a, k_first, k_end < full ? k_end : full, step);
+        if (k_first < full) // the first run past the full rows
+            k_first += (full - k_first + step - 1) / step * step;
+        if (k_first >= k_end)
+            return;
+    }
+    other_runs<CH, G, false>(a, k_first, k_end, step);
 }
 
 // Extraction of carrying rows r = r_first + i*r_step < min(r_end, R), any

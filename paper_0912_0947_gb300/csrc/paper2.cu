@@ -48,10 +48,6 @@ __device__ __forceinline__ void write_res(const P2Args &a, bool stats)
 }
 
 constexpr int kUnitThreads = 256; // at most 256: the staging area holds 8 warps
-constexpr int kUnitsPerThread = 1; // one channel
-
-// Units one thread takes per iteration of p2_embed_units.
-int units_per_thread(uint32_t channels) { return channels > 1 ? 1 : kUnitsPerThread; }
 
 // Out of place every unit of the image; in place the units with carrying
 // pixels.  Three or four channels run the two-stage copy pipeline
@@ -79,9 +75,8 @@ __global__ void __launch_bounds__(kUnitThreads, CH == 4 ? 2 : CH == 1 ? 5 : 3) p
             a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x, (uint32_t)a.f.nunits, gridDim.x * blockDim.x,
             changed, sse, stage);
     } else {
-        p2::units_embed<CH, STATS, kUnitsPerThread, INPLACE>(
-            a.v, a.f, blockIdx.x * blockDim.x * kUnitsPerThread + threadIdx.x, (uint32_t)a.f.nunits,
-            gridDim.x * blockDim.x * kUnitsPerThread, changed, sse);
+        p2::units_embed<CH, STATS, INPLACE>(a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x,
+                                            (uint32_t)a.f.nunits, gridDim.x * blockDim.x, changed, sse);
     }
     if (STATS)
         block_stats(changed, sse, a.res, a.slot);
@@ -184,11 +179,10 @@ const void *extract_units_kernel(uint32_t ch)
 } // namespace
 
 // Launches the unit kernel over a.f's units.
-static cudaError_t launch_units(const void *k, P2Args &a, uint32_t channels, bool stats,
-                                cudaStream_t s)
+static cudaError_t launch_units(const void *k, P2Args &a, bool stats, cudaStream_t s)
 {
     const int grid = persistent_grid(k, kUnitThreads, 0, kAnyCtas, a.f.nunits,
-                                     (uint64_t)kUnitThreads * units_per_thread(channels));
+                                     (uint64_t)kUnitThreads);
     void *args[] = {&a};
     return launch_counting(k, dim3(grid), dim3(kUnitThreads), args, 0, s, stats ? a.res : nullptr, a.slot);
 }
@@ -209,7 +203,7 @@ bool p2_embed_fused(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
     else
         k = stats ? units_kernel<true, false, false>(g.channels)
                   : units_kernel<false, false, false>(g.channels);
-    *err = launch_units(k, a, g.channels, stats, s);
+    *err = launch_units(k, a, stats, s);
     return true;
 }
 
@@ -226,7 +220,7 @@ cudaError_t p2_embed(const uint8_t *cover, uint8_t *stego, const stego_geom &g,
         // kernel): whole vectors instead of one byte access per plane byte
         const void *k = stats ? units_kernel<true, true, false>(g.channels)
                               : units_kernel<false, true, false>(g.channels);
-        return launch_units(k, a, g.channels, stats, s);
+        return launch_units(k, a, stats, s);
     }
     const void *k = stats ? (const void *)p2_embed_rows<true> : (const void *)p2_embed_rows<false>;
     const int grid = row_grid(k, sh, a.v.R);
