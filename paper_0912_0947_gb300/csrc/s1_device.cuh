@@ -112,10 +112,72 @@ __device__ __forceinline__ uint4 embed_vec16(const EmbedView &a, uint64_t v, con
     return o;
 }
 
-// 16-byte vectors v = v_first + i*step (+ u*blockDim.x for u < V), v < v_end,
-// of a job whose cover and stego are 16-byte aligned.  Each warp's 128-bit
-// load and store instructions cover 512 contiguous bytes.  With STATS the
-// changed-byte count (= squared error, see vec_changes) is added to both
+// One round of a job whose cover and stego are 16-byte aligned: 16-byte vectors v =
+// v0 + u*blockDim.x for u < V, v < v_end.  Each warp's 128-bit load and store
+// instructions cover 512 contiguous bytes.  With STATS the changed-byte count (=
+// squared error, see vec_changes) is added to n: a thread covers at most (bytes /
+// threads) bytes, far below 2^32 for any cover in device memory.
+template <int V, bool STATS>
+__device__ __forceinline__ void embed_vec_round(const EmbedView &a, uint64_t v0, uint64_t v_end,
+                                                uint32_t &n)
+{
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.cover);
+    uint4 *dst = reinterpret_cast<uint4 *>(a.stego);
+    // vectors [fast_lo, fast_hi) carry message bytes only (two per vector, a
+    // 16-bit load when the message is 2-byte aligned) in all 16 bytes
+    const uint64_t fast_lo = a.header ? 2u : 0u;
+    const uint64_t fast_hi = a.msg_even ? (a.t_bytes >> 4) : 0u;
+    const unsigned short *__restrict__ mw =
+        reinterpret_cast<const unsigned short *>(a.msg) - fast_lo;
+    uint4 c[V];
+    uint32_t p[V];
+    const uint64_t vlast = v0 + (uint64_t)(V - 1) * blockDim.x;
+    if (v0 >= fast_lo && vlast < fast_hi && vlast < v_end) {
+        // the whole round inside the message: no per-vector checks
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            c[u] = __ldcs(src + v0 + (uint64_t)u * blockDim.x);
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            p[u] = __ldg(mw + v0 + (uint64_t)u * blockDim.x);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+            const uint32_t r0 = __byte_perm(p[u], 0u, 0x0000u);
+            const uint32_t r1 = __byte_perm(p[u], 0u, 0x1111u);
+            uint4 o;
+            o.x = (c[u].x & 0xFEFEFEFEu) | spread_hi(r0);
+            o.y = (c[u].y & 0xFEFEFEFEu) | spread_lo(r0);
+            o.z = (c[u].z & 0xFEFEFEFEu) | spread_hi(r1);
+            o.w = (c[u].w & 0xFEFEFEFEu) | spread_lo(r1);
+            if (STATS)
+                n += vec_changes(o, c[u]);
+            __stcs(dst + v0 + (uint64_t)u * blockDim.x, o);
+        }
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        const uint64_t v = v0 + (uint64_t)u * blockDim.x;
+        if (v < v_end)
+            c[u] = __ldcs(src + v);
+    }
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        const uint64_t v = v0 + (uint64_t)u * blockDim.x;
+        p[u] = 0;
+        if (v < v_end && (v << 4) < a.t_bytes)
+            p[u] = stream_pair(a, v << 1);
+    }
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        const uint64_t v = v0 + (uint64_t)u * blockDim.x;
+        if (v >= v_end)
+            continue;
+        __stcs(dst + v, embed_vec16<STATS>(a, v, c[u], p[u], n));
+    }
+}
+
+// The rounds from v0 = v_first + i*step on, v0 < v_end; the count is added to both
 // accumulators.
 template <int V, bool STATS>
 __device__ __forceinline__ void embed_vec_range(const EmbedView &a, uint64_t v_first,
@@ -123,65 +185,9 @@ __device__ __forceinline__ void embed_vec_range(const EmbedView &a, uint64_t v_f
                                                 unsigned long long &changed,
                                                 unsigned long long &sse)
 {
-    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.cover);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.stego);
-    // changed bytes of this call in 32 bits: a thread covers at most
-    // (bytes / threads) bytes, far below 2^32 for any cover in device memory
     uint32_t n = 0;
-    // vectors [fast_lo, fast_hi) carry message bytes only (two per vector, a
-    // 16-bit load when the message is 2-byte aligned) in all 16 bytes
-    const uint64_t fast_lo = a.header ? 2u : 0u;
-    const uint64_t fast_hi = a.msg_even ? (a.t_bytes >> 4) : 0u;
-    const unsigned short *__restrict__ mw =
-        reinterpret_cast<const unsigned short *>(a.msg) - fast_lo;
-    for (uint64_t v0 = v_first; v0 < v_end; v0 += step) {
-        uint4 c[V];
-        uint32_t p[V];
-        const uint64_t vlast = v0 + (uint64_t)(V - 1) * blockDim.x;
-        if (v0 >= fast_lo && vlast < fast_hi && vlast < v_end) {
-            // the whole round inside the message: no per-vector checks
-#pragma unroll
-            for (int u = 0; u < V; ++u)
-                c[u] = __ldcs(src + v0 + (uint64_t)u * blockDim.x);
-#pragma unroll
-            for (int u = 0; u < V; ++u)
-                p[u] = __ldg(mw + v0 + (uint64_t)u * blockDim.x);
-#pragma unroll
-            for (int u = 0; u < V; ++u) {
-                const uint32_t r0 = __byte_perm(p[u], 0u, 0x0000u);
-                const uint32_t r1 = __byte_perm(p[u], 0u, 0x1111u);
-                uint4 o;
-                o.x = (c[u].x & 0xFEFEFEFEu) | spread_hi(r0);
-                o.y = (c[u].y & 0xFEFEFEFEu) | spread_lo(r0);
-                o.z = (c[u].z & 0xFEFEFEFEu) | spread_hi(r1);
-                o.w = (c[u].w & 0xFEFEFEFEu) | spread_lo(r1);
-                if (STATS)
-                    n += vec_changes(o, c[u]);
-                __stcs(dst + v0 + (uint64_t)u * blockDim.x, o);
-            }
-            continue;
-        }
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-            const uint64_t v = v0 + (uint64_t)u * blockDim.x;
-            if (v < v_end)
-                c[u] = __ldcs(src + v);
-        }
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-            const uint64_t v = v0 + (uint64_t)u * blockDim.x;
-            p[u] = 0;
-            if (v < v_end && (v << 4) < a.t_bytes)
-                p[u] = stream_pair(a, v << 1);
-        }
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-            const uint64_t v = v0 + (uint64_t)u * blockDim.x;
-            if (v >= v_end)
-                continue;
-            __stcs(dst + v, embed_vec16<STATS>(a, v, c[u], p[u], n));
-        }
-    }
+    for (uint64_t v0 = v_first; v0 < v_end; v0 += step)
+        embed_vec_round<V, STATS>(a, v0, v_end, n);
     if (STATS) {
         changed += n;
         sse += n;
@@ -291,74 +297,82 @@ __device__ __forceinline__ uint4 embed_vec16_at(const EmbedView &a, uint64_t k0,
     return o;
 }
 
-// Cover and stego with the same misalignment: h = (-cover) mod 16 head
-// bytes, then aligned vectors j at cover + h + 16j (j < j_end), each with
-// the stream bits of bytes h + 16j onwards.  Head and tail bytes are left to
-// the caller.
+// One round of a job whose cover and stego have the same misalignment: aligned
+// vectors j = j0 + u*blockDim.x for u < V, j < j_end, of cover + h + 16j (h head
+// bytes to an aligned address, left to the caller as the tail is), each with the
+// stream bits of bytes h + 16j onwards.  n as in embed_vec_round.
+template <int V, bool STATS>
+__device__ __forceinline__ void embed_shift_round(const EmbedView &a, uint32_t h, uint64_t j0,
+                                                  uint64_t j_end, uint32_t &n)
+{
+    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.cover + h);
+    uint4 *dst = reinterpret_cast<uint4 *>(a.stego + h);
+    // cover byte h + 16j carries stream bit h + 16j: stream byte h/8 + 2j
+    // (message byte m0 + 2j), cut at bit h % 8
+    const uintptr_t m0 = (uintptr_t)a.msg + (h >> 3) - (a.header ? 4u : 0u);
+    const uint32_t bsh = h & 7u;
+    uint4 c[V];
+    uint32_t p[V];
+    const uint64_t jl = j0 + (uint64_t)(V - 1) * blockDim.x;
+    if (jl < j_end && window_inner(a, h + (j0 << 4), h + (jl << 4))) {
+        // the whole round inside the message: no per-vector checks
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            c[u] = __ldcs(src + j0 + (uint64_t)u * blockDim.x);
+        // the V windows start 2 * blockDim.x message bytes apart, a
+        // multiple of 4: the same offset within an aligned word
+        const uintptr_t pm = m0 + 2u * j0;
+        const uint32_t *__restrict__ wp =
+            reinterpret_cast<const uint32_t *>(pm & ~(uintptr_t)3u);
+        const uint32_t wsh = 8u * (uint32_t)(pm & 3u);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+            const uint32_t *w = wp + (uint64_t)u * (blockDim.x >> 1);
+            p[u] = bits16_from(__funnelshift_r(__ldg(w), __ldg(w + 1), wsh), bsh);
+        }
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+            const uint4 o = spread16(c[u], p[u]);
+            if (STATS)
+                n += vec_changes(o, c[u]);
+            __stcs(dst + j0 + (uint64_t)u * blockDim.x, o);
+        }
+        return;
+    }
+    if (jl < j_end && h + (j0 << 4) >= a.t_bytes) {
+        // the whole round past the carrying bytes: a copy, all loads
+        // first
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            c[u] = __ldcs(src + j0 + (uint64_t)u * blockDim.x);
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            __stcs(dst + j0 + (uint64_t)u * blockDim.x, c[u]);
+        return;
+    }
+    // a round at an edge: one vector at a time, with the checks
+#pragma unroll 1
+    for (int u = 0; u < V; ++u) {
+        const uint64_t j = j0 + (uint64_t)u * blockDim.x;
+        if (j >= j_end)
+            break;
+        const uint64_t k0 = h + (j << 4);
+        const uint32_t pw = k0 < a.t_bytes ? stream_bits16(a, k0) : 0u;
+        __stcs(dst + j, embed_vec16_at<STATS>(a, k0, __ldcs(src + j), pw, n));
+    }
+}
+
+// The rounds from j0 = j_first + i*step on, j0 < j_end; the count is added to both
+// accumulators.
 template <int V, bool STATS>
 __device__ __forceinline__ void embed_shift_range(const EmbedView &a, uint32_t h,
                                                   uint64_t j_first, uint64_t j_end,
                                                   uint64_t step, unsigned long long &changed,
                                                   unsigned long long &sse)
 {
-    const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.cover + h);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.stego + h);
     uint32_t n = 0;
-    // cover byte h + 16j carries stream bit h + 16j: stream byte h/8 + 2j
-    // (message byte m0 + 2j), cut at bit h % 8
-    const uintptr_t m0 = (uintptr_t)a.msg + (h >> 3) - (a.header ? 4u : 0u);
-    const uint32_t bsh = h & 7u;
-    for (uint64_t j0 = j_first; j0 < j_end; j0 += step) {
-        uint4 c[V];
-        uint32_t p[V];
-        const uint64_t jl = j0 + (uint64_t)(V - 1) * blockDim.x;
-        if (jl < j_end && window_inner(a, h + (j0 << 4), h + (jl << 4))) {
-            // the whole round inside the message: no per-vector checks
-#pragma unroll
-            for (int u = 0; u < V; ++u)
-                c[u] = __ldcs(src + j0 + (uint64_t)u * blockDim.x);
-            // the V windows start 2 * blockDim.x message bytes apart, a
-            // multiple of 4: the same offset within an aligned word
-            const uintptr_t pm = m0 + 2u * j0;
-            const uint32_t *__restrict__ wp =
-                reinterpret_cast<const uint32_t *>(pm & ~(uintptr_t)3u);
-            const uint32_t wsh = 8u * (uint32_t)(pm & 3u);
-#pragma unroll
-            for (int u = 0; u < V; ++u) {
-                const uint32_t *w = wp + (uint64_t)u * (blockDim.x >> 1);
-                p[u] = bits16_from(__funnelshift_r(__ldg(w), __ldg(w + 1), wsh), bsh);
-            }
-#pragma unroll
-            for (int u = 0; u < V; ++u) {
-                const uint4 o = spread16(c[u], p[u]);
-                if (STATS)
-                    n += vec_changes(o, c[u]);
-                __stcs(dst + j0 + (uint64_t)u * blockDim.x, o);
-            }
-            continue;
-        }
-        if (jl < j_end && h + (j0 << 4) >= a.t_bytes) {
-            // the whole round past the carrying bytes: a copy, all loads
-            // first
-#pragma unroll
-            for (int u = 0; u < V; ++u)
-                c[u] = __ldcs(src + j0 + (uint64_t)u * blockDim.x);
-#pragma unroll
-            for (int u = 0; u < V; ++u)
-                __stcs(dst + j0 + (uint64_t)u * blockDim.x, c[u]);
-            continue;
-        }
-        // a round at an edge: one vector at a time, with the checks
-#pragma unroll 1
-        for (int u = 0; u < V; ++u) {
-            const uint64_t j = j0 + (uint64_t)u * blockDim.x;
-            if (j >= j_end)
-                break;
-            const uint64_t k0 = h + (j << 4);
-            const uint32_t pw = k0 < a.t_bytes ? stream_bits16(a, k0) : 0u;
-            __stcs(dst + j, embed_vec16_at<STATS>(a, k0, __ldcs(src + j), pw, n));
-        }
-    }
+    for (uint64_t j0 = j_first; j0 < j_end; j0 += step)
+        embed_shift_round<V, STATS>(a, h, j0, j_end, n);
     if (STATS) {
         changed += n;
         sse += n;

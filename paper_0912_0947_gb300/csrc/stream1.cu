@@ -59,11 +59,11 @@ __global__ void __launch_bounds__(512) embed_vec(EmbedArgs e)
     const uint64_t nvec = e.a.n_bytes >> 4;
     const uint32_t round = blockDim.x * V;
     const uint32_t ntiles = (uint32_t)((nvec + round - 1) / round);
+    uint32_t n = 0;
     for_tiles(e.slot, ntiles, [&](uint32_t tile) {
-        const uint64_t v0 = (uint64_t)tile * round;
-        s1::embed_vec_range<V, STATS>(e.a, v0 + threadIdx.x, v0 + round < nvec ? v0 + round : nvec,
-                                      round, changed, sse);
+        s1::embed_vec_round<V, STATS>(e.a, (uint64_t)tile * round + threadIdx.x, nvec, n);
     });
+    changed = sse = n;
     if (blockIdx.x == 0)
         s1::embed_tail<STATS>(e.a, changed, sse);
     if (STATS)
@@ -86,9 +86,10 @@ __device__ __forceinline__ void head_tail(const s1::EmbedView &a, uint32_t h, ui
     }
 }
 
-// Cover and stego with the same misalignment: aligned vectors after h head
-// bytes, the stream cut at bit h % 8; the last CTA does the head and the tail.
-// Requires n_bytes >= h.  Tiles as in embed_vec.
+// Cover and stego with the same misalignment (or none and a message at an odd
+// address, see kOddMsgShift): aligned vectors after h head bytes, the stream cut at
+// bit h % 8; the last CTA does the head and the tail.  Requires n_bytes >= h.  Tiles
+// as in embed_vec.
 template <int V, bool STATS>
 __global__ void __launch_bounds__(512) embed_shift(EmbedArgs e, uint32_t h)
 {
@@ -101,11 +102,12 @@ __global__ void __launch_bounds__(512) embed_shift(EmbedArgs e, uint32_t h)
     const uint32_t ntiles = (uint32_t)((nvb + round - 1) / round);
     if (blockIdx.x == gridDim.x - 1)
         head_tail<STATS>(e.a, h, nvb, changed, sse);
+    uint32_t n = 0;
     for_tiles(e.slot, ntiles, [&](uint32_t tile) {
-        const uint64_t j0 = (uint64_t)tile * round;
-        s1::embed_shift_range<V, STATS>(e.a, h, j0 + threadIdx.x, j0 + round < nvb ? j0 + round : nvb,
-                                        round, changed, sse);
+        s1::embed_shift_round<V, STATS>(e.a, h, (uint64_t)tile * round + threadIdx.x, nvb, n);
     });
+    changed += n;
+    sse += n;
     if (STATS)
         block_stats(changed, sse, e.res, e.slot);
     else
@@ -301,6 +303,12 @@ constexpr int kShiftV = 4;
 constexpr int kFunnelV = 4;
 constexpr int kExtractShiftV = 4;
 
+// Aligned covers and a message at an odd address, from these bytes on: embed_shift,
+// which cuts the stream from aligned message words at any address, where embed_vec
+// loads it byte by byte (8192x8192x3 85.0 us, by a stride 82.9; embed_shift 64.9;
+// 4096x3072x3 17.9 / 16.6; below, its head costs more: 1920x1080x3 6.8 / 7.9).
+constexpr uint64_t kOddMsgShift = 16u << 20;
+
 int clamp_vec(int v) { return (v == 1 || v == 2 || v == 8) ? v : 4; }
 
 // Threads of the misaligned embeds' CTAs at most: 3839x2159x3, both 13 bytes
@@ -342,7 +350,7 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
     if (aligned16(cover) && aligned16(stego) && bulk_stages(sh))
         return s1_embed_bulk(cover, stego, n_bytes, t_bytes, msg, slen, header, nbits, stats,
                              res, res_msg_bytes, sh, s, slot);
-    if (aligned16(cover) && aligned16(stego)) {
+    if (aligned16(cover) && aligned16(stego) && (e.a.msg_even || n_bytes < kOddMsgShift)) {
         const int vec = clamp_vec(sh.vec), T = sh.threads;
         const void *k = nullptr;
         switch (vec) {
