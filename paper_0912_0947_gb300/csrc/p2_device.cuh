@@ -340,9 +340,9 @@ __host__ __device__ constexpr uint32_t stage_vectors()
 // back by the same thread.  BATCHED: three channels' plane byte at unit byte 0 (see
 // plan_units' lead), and a unit's row by a division each: kept from unit to unit by
 // additions it costs registers that the batched kernels spill (300 HD frames 645 us,
-// so 626; one channel in the single-cover kernel, which does not spill, 31.0
-// and 32.1).
-template <int CH, bool STATS, bool INPLACE = false, bool BATCHED = false>
+// so 624; one channel in the single-cover kernel, which does not spill, 31.0
+// and 32.1).  SHIFTED = false: the addresses agree mod 16 (f.d = 0).
+template <int CH, bool STATS, bool INPLACE = false, bool BATCHED = false, bool SHIFTED = true>
 __device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32_t k_first,
                                             uint32_t k_end, uint32_t step,
                                             unsigned long long &changed, unsigned long long &sse)
@@ -364,7 +364,7 @@ __device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32
 #pragma unroll
         for (int q = 0; q < CH; ++q)
             set_vec(c, q, __ldcs(src + (uint64_t)k * CH + q));
-        if (!INPLACE && f.d)
+        if (SHIFTED && !INPLACE && f.d)
             set_vec(c, CH, __ldcs(src + (uint64_t)k * CH + CH));
         if constexpr (BATCHED) {
             const uint64_t x = f.x0 + 16ull * k;
@@ -373,7 +373,7 @@ __device__ __forceinline__ void units_embed(const View &a, const Flat &f, uint32
         }
         UnitJob J;
         plan_unit(a, k < carry, r, col, J);
-        if (!INPLACE && f.d) {
+        if (SHIFTED && !INPLACE && f.d) {
             join_unit<CH>(c, f.d, o);
         } else {
 #pragma unroll
@@ -681,18 +681,22 @@ __device__ __forceinline__ void get_pairs(const uint32_t (&w)[4 * CH], uint32_t 
 // quarters' vectors at a time.  BATCHED: a run's row and block by a 32-bit division,
 // else kept by additions (8192x8192x3 33.1 us, 33.4 by divisions; in the batched
 // kernel the additions cost registers that it spills: 1024 paper covers 380 us, by
-// divisions here and in other_runs 372).
+// divisions here and in other_runs 372), the step in rows and blocks found when there
+// is a next run: a launch of one run per thread is a chain of latencies, in which
+// that division and one for the first run after these were 0.4 of 2.0 us (gray
+// 1920x1080).  Returns the first k that it did not take.
 template <int CH, int PLANE, int GA, bool BATCHED>
-__device__ __forceinline__ void full_runs(const View &a, uint64_t k_first, uint64_t k_end,
+__device__ __forceinline__ uint64_t full_runs(const View &a, uint64_t k_first, uint64_t k_end,
                                           uint32_t step)
 {
     const uint32_t rpr = a.Q / 16u, W16 = a.W / 16u;
     const uint32_t stride = rpr * CH; // vectors from quarter to quarter
     uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
-    const uint32_t dr = step / rpr, db = step - dr * rpr;
+    uint32_t dr = 0, db = 0; // (step > 0: not both, once known)
     const uint4 *__restrict__ src = reinterpret_cast<const uint4 *>(a.src);
     uint4 *out = reinterpret_cast<uint4 *>(a.msg_out);
-    for (uint64_t k = k_first; k < k_end; k += step) {
+    uint64_t k = k_first;
+    while (k < k_end) {
         if constexpr (BATCHED) {
             r = row_of(k, rpr);
             b = (uint32_t)(k - (uint64_t)r * rpr);
@@ -723,9 +727,18 @@ __device__ __forceinline__ void full_runs(const View &a, uint64_t k_first, uint6
             }
         }
         out[k] = make_uint4(M[0], M[1], M[2], M[3]);
-        if constexpr (!BATCHED)
+        k += step;
+        if constexpr (!BATCHED) {
+            if (k >= k_end)
+                break;
+            if ((dr | db) == 0) {
+                dr = step / rpr;
+                db = step - dr * rpr;
+            }
             rc_add(r, b, dr, db, rpr);
+        }
     }
+    return k;
 }
 
 // Runs k = k_first + i*step < k_end of any layout, G quarters' vectors at a time
@@ -736,7 +749,7 @@ __device__ __forceinline__ void other_runs(const View &a, uint64_t k_first, uint
 {
     const uint32_t rpr = run_row(a);
     uint32_t r = row_of(k_first, rpr), b = (uint32_t)(k_first - (uint64_t)r * rpr);
-    const uint32_t dr = step / rpr, db = step - dr * rpr;
+    uint32_t dr = 0, db = 0;
     const uint64_t C = (uint64_t)a.W * a.H * CH;
     for (uint64_t k = k_first; k < k_end; k += step) {
         if constexpr (BATCHED) {
@@ -771,8 +784,15 @@ __device__ __forceinline__ void other_runs(const View &a, uint64_t k_first, uint
                 }
             }
         }
-        if constexpr (!BATCHED)
+        if constexpr (!BATCHED) {
+            if (k + step >= k_end)
+                break;
+            if ((dr | db) == 0) {
+                dr = step / rpr;
+                db = step - dr * rpr;
+            }
             rc_add(r, b, dr, db, rpr);
+        }
     }
 }
 
@@ -782,17 +802,16 @@ __host__ __device__ inline uint64_t aligned_full_runs(const View &a)
     return (uint64_t)(a.L_last == a.Q ? a.R : a.R - 1) * (a.Q / 16u);
 }
 
-// Runs k = k_first + i*step < k_end of an aligned layout's full rows, GA quarters'
-// vectors at a time.
+// full_runs of the cover's plane.
 template <int CH, int GA, bool BATCHED>
-__device__ __forceinline__ void aligned_runs(const View &a, uint64_t k_first, uint64_t k_end,
+__device__ __forceinline__ uint64_t aligned_runs(const View &a, uint64_t k_first, uint64_t k_end,
                                              uint32_t step)
 {
     switch (CH == 1 ? 0u : a.plane) {
-    case 0: full_runs<CH, 0, GA, BATCHED>(a, k_first, k_end, step); break;
-    case 1: full_runs<CH, CH == 1 ? 0 : 1, GA, BATCHED>(a, k_first, k_end, step); break;
-    case 2: full_runs<CH, CH == 1 ? 0 : 2, GA, BATCHED>(a, k_first, k_end, step); break;
-    default: full_runs<CH, CH == 4 ? 3 : 0, GA, BATCHED>(a, k_first, k_end, step); break;
+    case 0: return full_runs<CH, 0, GA, BATCHED>(a, k_first, k_end, step);
+    case 1: return full_runs<CH, CH == 1 ? 0 : 1, GA, BATCHED>(a, k_first, k_end, step);
+    case 2: return full_runs<CH, CH == 1 ? 0 : 2, GA, BATCHED>(a, k_first, k_end, step);
+    default: return full_runs<CH, CH == 4 ? 3 : 0, GA, BATCHED>(a, k_first, k_end, step);
     }
 }
 
@@ -806,9 +825,7 @@ __device__ __forceinline__ void runs_extract(const View &a, uint64_t k_first, ui
         return;
     if (runs_aligned(a)) {
         const uint64_t full = aligned_full_runs(a);
-        aligned_runs<CH, GA, false>(a, k_first, k_end < full ? k_end : full, step);
-        if (k_first < full) // the first run past the full rows
-            k_first += (full - k_first + step - 1) / step * step;
+        k_first = aligned_runs<CH, GA, false>(a, k_first, k_end < full ? k_end : full, step);
         if (k_first >= k_end)
             return;
     }

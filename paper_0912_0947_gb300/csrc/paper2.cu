@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kUnitThreads, CH == 4 ? 2 : CH == 1 ? 5 : 3) p
             a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x, (uint32_t)a.f.nunits, gridDim.x * blockDim.x,
             changed, sse, stage);
     } else {
-        p2::units_embed<CH, STATS, INPLACE>(a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x,
+        p2::units_embed<CH, STATS, INPLACE, false, SHIFTED>(a.v, a.f, blockIdx.x * blockDim.x + threadIdx.x,
                                             (uint32_t)a.f.nunits, gridDim.x * blockDim.x, changed, sse);
     }
     if (STATS)
@@ -153,7 +153,7 @@ template <bool STATS, bool INPLACE, bool SHIFTED>
 const void *units_kernel(uint32_t ch)
 {
     switch (ch) {
-    case 1: return (const void *)p2_embed_units<1, STATS, INPLACE, false>;
+    case 1: return (const void *)p2_embed_units<1, STATS, INPLACE, SHIFTED>;
     case 3: return (const void *)p2_embed_units<3, STATS, INPLACE, SHIFTED>;
     default: return (const void *)p2_embed_units<4, STATS, INPLACE, SHIFTED>;
     }
