@@ -251,18 +251,12 @@ __device__ __forceinline__ uint32_t unit_fields(uint64_t X, int i)
         // stream bytes 2i, 2i+1; lanes take high nibble, low nibble, high, low
         const uint32_t r = __byte_perm(i < 2 ? hi : lo, 0u, (i & 1) ? 0x0011u : 0x2233u);
         return ((r >> 4) & 0x000F000Fu) | (r & 0x0F000F00u);
-    } else if constexpr (K == 3) {
+    } else {
+        static_assert(K == 3, "one to four bits per byte");
         const uint32_t h = i < 2 ? hi : lo;
         const uint32_t t = (i & 1) ? (h & 0xFFFu) : (h >> 12);
         const uint32_t p = t * 0x01000004u;
         return (p & 0x07000700u) | ((p & 0x38003800u) >> 11);
-    } else {
-        constexpr uint32_t MASK = (1u << K) - 1u;
-        uint32_t f = 0;
-#pragma unroll
-        for (int l = 0; l < 4; ++l)
-            f |= (uint32_t)((X >> (64 - K * (4 * i + l + 1))) & MASK) << (8 * l);
-        return f;
     }
 }
 
@@ -284,7 +278,8 @@ __device__ __forceinline__ uint64_t unit_window(const uint32_t (&g)[4])
         for (int i = 0; i < 4; ++i) // lane l -> bits 30-2l, 31-2l of the product
             hi |= (((g[i] & 0x03030303u) * 0x40100401u) >> 24) << (24 - 8 * i);
         return (uint64_t)hi << 32;
-    } else if constexpr (K == 4) {
+    } else {
+        static_assert(K == 4, "k = 3: unit_window3");
         uint32_t b[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -294,13 +289,6 @@ __device__ __forceinline__ uint64_t unit_window(const uint32_t (&g)[4])
         const uint32_t hi = __byte_perm(b[0], b[1], 0x0246u); // b0.l0 b0.l2 b1.l0 b1.l2, first on top
         const uint32_t lo = __byte_perm(b[2], b[3], 0x0246u);
         return ((uint64_t)hi << 32) | lo;
-    } else {
-        constexpr uint32_t MASK = (1u << K) - 1u;
-        uint64_t X = 0;
-#pragma unroll
-        for (int t = 0; t < 16; ++t)
-            X |= (uint64_t)((g[t >> 2] >> (8 * (t & 3))) & MASK) << (64 - K * (t + 1));
-        return X;
     }
 }
 
@@ -751,41 +739,41 @@ __global__ void __launch_bounds__(512) extractk_units(KView a)
     }
     if constexpr (K == 3) {
         extract3_units<CH, FLAT>(a, ulo, nunits, hb, sbytes);
-        return;
-    }
-    constexpr int U = units_per_iter<CH>();
-    for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x * U + threadIdx.x; v0 < nunits;
-         v0 += (uint64_t)gridDim.x * blockDim.x * U) {
-        uint32_t w[U][4 * CH];
+    } else {
+        constexpr int U = units_per_iter<CH>();
+        for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x * U + threadIdx.x; v0 < nunits;
+             v0 += (uint64_t)gridDim.x * blockDim.x * U) {
+            uint32_t w[U][4 * CH];
 #pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const uint64_t u = v0 + (uint64_t)r * blockDim.x;
-            if (u < nunits && (!FLAT || u >= ulo))
-                read_unit<CH, FLAT>(a, u, w[r]);
-        }
+            for (int r = 0; r < U; ++r) {
+                const uint64_t u = v0 + (uint64_t)r * blockDim.x;
+                if (u < nunits && (!FLAT || u >= ulo))
+                    read_unit<CH, FLAT>(a, u, w[r]);
+            }
 #pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const uint64_t u = v0 + (uint64_t)r * blockDim.x;
-            if (u >= nunits || (FLAT && u < ulo))
-                continue;
-            uint32_t g[4];
-            get_unit<CH>(w[r], a.f.sel, g);
-            const uint64_t X = unit_window<K>(g);
-            const uint64_t q0 = 2u * K * u; // first stream byte of the unit
-            uint8_t *op = a.out + (q0 - hb);
-            if ((K & 1) == 0 && q0 >= hb && q0 + 2 * K <= sbytes &&
-                (((uintptr_t)op & 3u) == 0)) {
-                // message bytes only, 4-byte aligned: K/2 word stores
+            for (int r = 0; r < U; ++r) {
+                const uint64_t u = v0 + (uint64_t)r * blockDim.x;
+                if (u >= nunits || (FLAT && u < ulo))
+                    continue;
+                uint32_t g[4];
+                get_unit<CH>(w[r], a.f.sel, g);
+                const uint64_t X = unit_window<K>(g);
+                const uint64_t q0 = 2u * K * u; // first stream byte of the unit
+                uint8_t *op = a.out + (q0 - hb);
+                if ((K & 1) == 0 && q0 >= hb && q0 + 2 * K <= sbytes &&
+                    (((uintptr_t)op & 3u) == 0)) {
+                    // message bytes only, 4-byte aligned: K/2 word stores
 #pragma unroll
-                for (int i = 0; i < K / 2; ++i)
-                    reinterpret_cast<uint32_t *>(op)[i] =
-                        __byte_perm((uint32_t)(X >> (32 - 32 * i)), 0u, 0x0123u);
-            } else {
+                    for (int i = 0; i < K / 2; ++i)
+                        reinterpret_cast<uint32_t *>(op)[i] =
+                            __byte_perm((uint32_t)(X >> (32 - 32 * i)), 0u, 0x0123u);
+                } else {
 #pragma unroll
-                for (int i = 0; i < 2 * K; ++i) {
-                    const uint64_t q = q0 + i; // stream byte
-                    if (q >= hb && q < sbytes)
-                        a.out[q - hb] = (uint8_t)(X >> (56 - 8 * i));
+                    for (int i = 0; i < 2 * K; ++i) {
+                        const uint64_t q = q0 + i; // stream byte
+                        if (q >= hb && q < sbytes)
+                            a.out[q - hb] = (uint8_t)(X >> (56 - 8 * i));
+                    }
                 }
             }
         }
