@@ -364,11 +364,11 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
                                          (uint64_t)T * vec);
         return launch_tiles(k, grid, T, args, e, stats, (nvec + T * vec - 1) / (T * vec), s);
     }
-    // heads up to a 128-byte boundary of the stego, so that a warp's vectors are
-    // whole cache lines (16-byte boundaries in a small cover)
+    // heads up to a 128-byte boundary of the stego, so that a warp stores whole cache
+    // lines (16-byte boundaries in a small cover)
     const int T = sh.threads < kShiftThreads ? sh.threads : kShiftThreads;
     const uint32_t line = n_bytes >= 16384u ? 127u : 15u;
-    const uint32_t h = (uint32_t)(-(uintptr_t)cover & line);
+    const uint32_t h = (uint32_t)(-(uintptr_t)stego & line);
     if ((((uintptr_t)cover ^ (uintptr_t)stego) & 15u) == 0 && n_bytes >= (uint64_t)h + 16u) {
         const void *k = stats ? (const void *)embed_shift<kShiftV, true>
                               : (const void *)embed_shift<kShiftV, false>;
@@ -377,9 +377,8 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         void *sargs[] = {&e, (void *)&h};
         return launch_tiles(k, grid, T, sargs, e, stats, (nvb + T * kShiftV - 1) / (T * kShiftV), s);
     }
-    const uint32_t hs = (uint32_t)(-(uintptr_t)stego & line);
-    if (cover != stego && n_bytes >= (uint64_t)hs + 16u) {
-        const uint32_t d = (uint32_t)(((uintptr_t)cover + hs) & 15u), b = d & 3u;
+    if (cover != stego && n_bytes >= (uint64_t)h + 16u) {
+        const uint32_t d = (uint32_t)(((uintptr_t)cover + h) & 15u), b = d & 3u;
         const uint32_t sel = b | ((b + 1) << 4) | ((b + 2) << 8) | ((b + 3) << 12);
         const void *k;
         constexpr int F = kFunnelV;
@@ -389,9 +388,9 @@ cudaError_t s1_embed(const uint8_t *cover, uint8_t *stego, uint64_t n_bytes, uin
         case 2: k = stats ? (const void *)embed_funnel<2, F, true> : (const void *)embed_funnel<2, F, false>; break;
         default: k = stats ? (const void *)embed_funnel<3, F, true> : (const void *)embed_funnel<3, F, false>; break;
         }
-        const uint64_t nvb = (n_bytes - hs) >> 4;
+        const uint64_t nvb = (n_bytes - h) >> 4;
         const int grid = persistent_grid(k, T, 0, sh.ctas_per_sm, nvb, (uint64_t)T * F);
-        void *fargs[] = {&e, (void *)&hs, (void *)&sel};
+        void *fargs[] = {&e, (void *)&h, (void *)&sel};
         return launch_tiles(k, grid, T, fargs, e, stats, (nvb + T * F - 1) / (T * F), s);
     }
     const void *k = stats ? (const void *)embed_bytes<true> : (const void *)embed_bytes<false>;
