@@ -51,8 +51,11 @@
  *     case the message buffer is not written.  STEGO_E_CUDA means a CUDA
  *     launch or memset failed (see cudaGetLastError in the caller's runtime).
  *   - Any byte alignment is accepted.  Cover and stego buffers that start on
- *     16-byte boundaries take the shortest path; all others run in whole
- *     vectors too, joined from the aligned ones around them.
+ *     16-byte boundaries take the shortest path; others run in whole vectors
+ *     too, joined from the aligned ones around them, except one plane or the
+ *     paper's layout of two or more than four channels, one plane in place at
+ *     an odd address and the paper's layout in place with rows that are not
+ *     whole 16-byte vectors, which go byte by byte.
  *   - In-place embedding (d_stego == d_cover) is allowed and then bytes past
  *     the embedded bits are not written.  Any other overlap between the
  *     buffers of one call is STEGO_E_INVAL.
@@ -211,16 +214,23 @@ int stego_capacity(uint64_t cover_bytes, const stego_geom *geom, uint32_t flags,
 /* Embed (Section VI).  Writes cover_bytes bytes of d_stego (out of place) or,
  * in place, the T = 8*|S| carrying bytes (STREAM1) / the 4*msg_bytes plane
  * bytes (PAPER2; with 1, 3 or 4 channels, rows of whole 16-byte vectors and
- * a 16-byte aligned buffer whole 16-pixel groups are rewritten, the bytes
- * outside the plane's carrying bytes with their own values: those groups
- * holding carrying pixels, in a batched call every group of the carrying
- * rows).  Bytes that do not carry the message keep their values.
+ * a 16-byte aligned buffer whole groups of 16 consecutive pixels are rewritten,
+ * the bytes outside the plane's carrying bytes with their own values: the
+ * groups that hold carrying pixels; a group may begin or end inside a row).
+ * Bytes that do not carry the message keep their values.
  *   d_cover, d_stego  cover and output image, cover_bytes each.
  *   d_msg, msg_bytes  message (may be NULL when msg_bytes == 0).
  *   geom              PAPER2 geometry (host pointer) or NULL for STREAM1.
  *   flags             layout | STEGO_HEADER_BE32 (STREAM1) | STEGO_FUSE_STATS.
  *   d_result          optional; required with STEGO_FUSE_STATS.  Filled with
  *                     changed/sse (if fused), msg_bytes and status STEGO_OK.
+ * Statistics go through one of 256 slots per device that belong to the streams
+ * they were first asked for on (stego_changed_bytes: 256 of its own); on further
+ * streams and under capture the result is zeroed by a memset first, and the kernel
+ * is launched in the ordinary way.  A queue of 300 streams, each a 256 MB copy, such
+ * a memset and an embed then launched as a programmatic dependent, has stopped
+ * making progress, cause unknown: do not fill hundreds of streams at once with
+ * embeds that wait for long copies.
  * Synchronous errors: STEGO_E_INVAL, STEGO_E_CAPACITY (message too long for
  * the cover; nothing written), STEGO_E_CUDA. */
 int stego_embed(const uint8_t *d_cover, uint8_t *d_stego, uint64_t cover_bytes,

@@ -511,7 +511,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_batch(const stego_desc *des
 // all of them on the CTA's path between two claims.  Per call, device time,
 // halving against this: 256 covers of sides 64 to 512 embed 24.4 -> 23.0 us,
 // extract 19.0 -> 16.7; 4096 uneven covers embed 2459 -> 2441; 1024 paper covers
-// 900 -> 896 and 392 -> 388; 300 HD paper frames extract 190 -> 188.
+// 900 -> 896 and 392 -> 388; 300 HD paper frames extract 190 -> 188 (all before the
+// paper kernels found rows by divisions).
 __device__ __forceinline__ uint32_t owner_of(const unsigned long long *start, uint32_t n,
                                              unsigned long long t)
 {
@@ -697,10 +698,11 @@ __device__ __forceinline__ void paper_embed_tile(const stego_desc &D, const Desc
             return; // a part past the tile's or the cover's end
         const uint32_t k0 = (uint32_t)b0 + threadIdx.x;
         const uint32_t k1 = (uint32_t)(b1 < inf.n_bytes ? b1 : inf.n_bytes);
-        // one unit per thread, loaded by the thread itself: under the
-        // 80-register cap a form staged through shared memory spilled more
-        // and ran slower (600 video frames: 1.53 against 1.26 ms), and so did
-        // the cp.async pipeline of the single-cover kernel (1.34-1.83 ms)
+        // one unit per thread, loaded by the thread itself: when these kernels
+        // had 80 registers and three CTAs per SM, a form staged through shared
+        // memory spilled more and ran slower (600 video frames: 1.53 against
+        // 1.26 ms), and so did the cp.async pipeline of the single-cover kernel
+        // (1.34-1.83 ms; 256 large RGB covers at 64 registers 3187 against 2545 us)
         switch (inf.channels) {
         case 1: p2::units_embed<1, STATS, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
         case 3: p2::units_embed<3, STATS, false, true>(job.v, job.f, k0, k1, blockDim.x, changed, sse); break;
@@ -1318,7 +1320,7 @@ extern "C" int stego_embed_batched_noalloc(const stego_desc *d_descs, uint32_t n
     const int st = noalloc_scratch(&ws);
     if (st != STEGO_OK)
         return st;
-    // the prep and scan launches rewrite every scratch word the persistent
-    // kernel reads, so the previous call's contents need no clearing
+    // the preparation launch rewrites every scratch word the persistent
+    // kernels read, so the previous call's contents need no clearing
     return stego::batched<true>(d_descs, n, d_results, flags, tune, ws, kNoAllocBytes, stream);
 }

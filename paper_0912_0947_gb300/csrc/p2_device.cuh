@@ -10,10 +10,12 @@
 // pairs back (Section VII step 6).
 //
 // Work units:
-//   unit  16 * CH consecutive stego bytes from a 16-byte boundary on (CH in
-//         {1,3,4} channels): CH whole vectors, which hold the plane bytes of
-//         16 consecutive pixels at the same unit bytes everywhere, whatever the row length and the buffers' addresses (see
-//         Flat).  One-pass out-of-place embedding (2C + N bytes).
+//   unit  16 * CH consecutive stego bytes, counted from a 128-byte boundary on
+//         (a 16-byte one in an image of less than 16 KiB; CH in {1,3,4}
+//         channels): CH whole vectors, which hold the plane bytes of 16
+//         consecutive pixels at the same unit bytes everywhere, whatever the
+//         row length and the buffers' addresses (see Flat).  One-pass
+//         out-of-place embedding (2C + N bytes).
 //   run   the message bytes of one row in one 16-byte block of the output:
 //         extraction reads the 16 pixels at columns i*L + j of each quarter
 //         i as the aligned vectors around them and ORs their pairs.

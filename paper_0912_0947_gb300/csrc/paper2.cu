@@ -4,7 +4,7 @@
 // per-row routines live in p2_device.cuh and are shared with the batched
 // kernels.
 //   p2_embed_units<CH,STATS,INPLACE,SHIFTED>  persistent grid over flat
-//       units (16*CH stego bytes from a 16-byte boundary on); 256-thread CTAs,
+//       units (16*CH stego bytes, see Flat); 256-thread CTAs,
 //       each warp's units copied to shared memory one iteration ahead
 //       (cp.async).  Out of place one pass (2C + N bytes) for any row length
 //       and any addresses; in place the units with carrying pixels, read and
@@ -59,7 +59,10 @@ constexpr int kUnitThreads = 256; // at most 256: the staging area holds 8 warps
 // pass over its units, so that short rows are bound by instructions.  Rows
 // that are not whole vectors took a copy and one thread per plane byte before:
 // 5471x3647x3 47.5 -> 24.1 us, one channel 28.3 -> 16.4, four 65.9 -> 31.1,
-// cover 3 bytes past a boundary 53.6 -> 25.4.
+// cover 3 bytes past a boundary 53.6 -> 25.4.  Whole-vector rows of one channel lose
+// where there are no statistics (8192x8192 23.6 -> 26.4 us; with them 28.9 as
+// before): neither more units in flight (26.4-28), other CTAs (26.1-28) nor a
+// kernel of their own for aligned addresses wins it back.
 template <int CH, bool STATS, bool INPLACE, bool SHIFTED>
 __global__ void __launch_bounds__(kUnitThreads, CH == 4 ? 2 : CH == 1 ? 5 : 3) p2_embed_units(P2Args a)
 {

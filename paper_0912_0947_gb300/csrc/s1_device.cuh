@@ -432,8 +432,8 @@ static __device__ __noinline__ uint32_t funnel_edge_vec(const EmbedView &a, uint
 }
 
 // Cover and stego at different addresses mod 16 (out of place, n_bytes =
-// C): h = (-stego) mod 16 head bytes, then aligned stego vectors j at stego
-// + h + 16j (j_lo <= j < j_hi).  The cover bytes of vector j, h + 16j .. h +
+// C): h head bytes up to an aligned address of the stego, left to the caller, then
+// aligned stego vectors j at stego + h + 16j (j_lo <= j < j_hi).  The cover bytes of vector j, h + 16j .. h +
 // 16j + 15, start at byte d = (cover + h) mod 16 = 4Q + (sel's b) of the
 // aligned cover vector A[j] at or below them: they are A[j]'s last 16 - d
 // bytes and A[j + 1]'s first d, joined by funnel16.

@@ -8,7 +8,8 @@
 // place an embed moves 2C + T/8 bytes, in place 2T + T/8, an extract T + T/8
 // (T = carrying bytes).  Each byte is read once and written once, so nothing
 // is staged through shared memory: 128-bit streaming loads/stores with V
-// vectors in flight per thread over a persistent grid feed HBM directly.
+// vectors in flight per thread feed HBM directly, over a persistent grid
+// (extracts of a known length: one round per CTA).
 // Misaligned buffers: cover and stego with the same address mod 16 run
 // aligned vectors after a head of scalar bytes (the stream cut at the head's
 // bit offset); cover and stego at different addresses mod 16 build each
